@@ -271,11 +271,10 @@ __global__ void __launch_bounds__(kBlock, 2) k_decide(NetDesc net, State st, int
   phase_decide<ZT, MIXED>(net, st, l, sm, dsm, mw);
 }
 
-template <typename ZT>
 __global__ void __launch_bounds__(kBlock) k_scan0(NetDesc net, State st, int l) {
   __shared__ Smem sm;
   if (cta_stopped(st)) return;
-  phase_scan0<ZT>(net, st, l, sm);
+  phase_scan0(net, st, l, sm);
 }
 
 template <typename ZT, bool MIXED>
@@ -288,16 +287,9 @@ __global__ void __launch_bounds__(kBlock, 2) k_step(NetDesc net, State st, int l
   phase_step<ZT, MIXED>(net, st, l, i, sm, dsm, mw);
 }
 
-template <typename ZT>
-__global__ void __launch_bounds__(kBlock) k_pack(NetDesc net, State st, int l) {
-  if (cta_stopped(st)) return;
-  phase_pack<ZT>(net, st, l);
-}
-
 // The neuron loop of layer l in one cooperative launch: the layer-start
 // decisions and first edge scan (prologue = 1; a launch that resumes after a
-// capacity halt skips them), one grid barrier per neuron step, and the
-// packing of the layer's sign codes.
+// capacity halt skips them) and one grid barrier per neuron step.
 template <typename ZT, bool MIXED>
 __global__ void __launch_bounds__(kBlock, 2) k_layer(NetDesc net, State st, int l, int i_begin, int prologue,
                                                      int mw) {
@@ -312,7 +304,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_layer(NetDesc net, State st, int 
     phase_decide<ZT, MIXED>(net, st, l, sm, dsm, mw);
     if (!grid_barrier(st.g, passed)) return;  // uniform per CTA
     if (cta_stopped(st)) return;
-    phase_scan0<ZT>(net, st, l, sm);
+    phase_scan0(net, st, l, sm);
     if (!grid_barrier(st.g, passed)) return;
     if (cta_stopped(st)) return;
   }
@@ -321,7 +313,6 @@ __global__ void __launch_bounds__(kBlock, 2) k_layer(NetDesc net, State st, int 
     if (!grid_barrier(st.g, passed)) return;
     if (cta_stopped(st)) return;
   }
-  phase_pack<ZT>(net, st, l);
 }
 
 // Exact check of every pairing made by fingerprint (deferred mode), after
@@ -496,9 +487,9 @@ static void realloc_state(pc_ctx* c, long long V, long long E, long long T, bool
   A(nb.exc, sizeof(float) * V);
   A(nb.SIG, sizeof(uint64_t) * S * V);
   A(nb.E, sizeof(int32_t) * 2 * E);
-  A(nb.list0, sizeof(int4) * E);
-  A(nb.list1, sizeof(int4) * E);
-  A(nb.flags, sizeof(uint32_t) * 2 * (E / 32));
+  A(nb.list0, sizeof(int32_t) * 3 * E);
+  A(nb.list1, sizeof(int32_t) * 3 * E);
+  A(nb.nx, sizeof(uint16_t) * E);
   A(nb.vlist, sizeof(int4) * E);
   A(nb.table, 32 * T);
   if (c->opt.keep_tape) {
@@ -506,7 +497,6 @@ static void realloc_state(pc_ctx* c, long long V, long long E, long long T, bool
     A(nb.tape_t, sizeof(double) * V);
   }
   PC_CUDA(cudaMemsetAsync(nb.table, 0xff, 32 * T, c->stream));
-  PC_CUDA(cudaMemsetAsync(nb.flags, 0, sizeof(uint32_t) * 2 * (E / 32), c->stream));
   StateBufs& ob = c->bufs;
   if (copy && ob.X) {
     const long long oV = c->Vcap, oE = c->Ecap, nV = std::min(oV, V), nE = std::min(oE, E);
@@ -520,10 +510,10 @@ static void realloc_state(pc_ctx* c, long long V, long long E, long long T, bool
     cp2(nb.SIG, 8 * V, ob.SIG, 8 * oV, 8 * nV, S);
     cp2(nb.E, 4 * E, ob.E, 4 * oE, 4 * nE, 2);
     cp2(nb.vlist, 16 * E, ob.vlist, 16 * oE, 16 * nE, 1);
-    // the splitting edges (and their flags) of the step that resumes
-    cp2(nb.list0, 16 * E, ob.list0, 16 * oE, 16 * nE, 1);
-    cp2(nb.list1, 16 * E, ob.list1, 16 * oE, 16 * nE, 1);
-    cp2(nb.flags, 4 * (E / 32), ob.flags, 4 * (oE / 32), 4 * (nE / 32), 2);
+    // the splitting edges of the step that resumes, and every edge's next crossing
+    cp2(nb.list0, 4 * E, ob.list0, 4 * oE, 4 * nE, 3);
+    cp2(nb.list1, 4 * E, ob.list1, 4 * oE, 4 * nE, 3);
+    cp2(nb.nx, 2 * E, ob.nx, 2 * oE, 2 * nE, 1);
     if (c->opt.keep_tape && ob.tape_pq) {
       cp2(nb.tape_pq, 4 * V, ob.tape_pq, 4 * oV, 4 * nV, 2);
       cp2(nb.tape_t, 8 * V, ob.tape_t, 8 * oV, 8 * nV, 1);
@@ -582,10 +572,9 @@ static State make_state(pc_ctx* c) {
   s.SIG = static_cast<uint64_t*>(c->bufs.SIG);
   s.EU = static_cast<int32_t*>(c->bufs.E);
   s.EW = s.EU + c->Ecap;
-  s.list[0] = static_cast<int4*>(c->bufs.list0);
-  s.list[1] = static_cast<int4*>(c->bufs.list1);
-  s.flags[0] = static_cast<uint32_t*>(c->bufs.flags);
-  s.flags[1] = s.flags[0] + (c->Ecap + 31) / 32;
+  s.list[0] = static_cast<int32_t*>(c->bufs.list0);
+  s.list[1] = static_cast<int32_t*>(c->bufs.list1);
+  s.nx = static_cast<uint16_t*>(c->bufs.nx);
   s.table = static_cast<uint64_t*>(c->bufs.table);
   s.vlist = static_cast<int4*>(c->bufs.vlist);
   s.deferred = c->deferred;
@@ -659,7 +648,7 @@ struct Kernels {
       if (prologue) {
         k_decide<ZT, MIXED><<<gs, kBlock, c->res_smem, c->stream>>>(c->net, st, l, c->mw);
         PC_CUDA(cudaGetLastError());
-        k_scan0<ZT><<<gs, kBlock, 0, c->stream>>>(c->net, st, l);
+        k_scan0<<<gs, kBlock, 0, c->stream>>>(c->net, st, l);
         PC_CUDA(cudaGetLastError());
         c->launches += 2;
       }
@@ -668,9 +657,6 @@ struct Kernels {
         PC_CUDA(cudaGetLastError());
         c->launches += 1;
       }
-      k_pack<ZT><<<gs, kBlock, 0, c->stream>>>(c->net, st, l);
-      PC_CUDA(cudaGetLastError());
-      c->launches += 1;
     }
   }
   static int occupancy(pc_ctx* c) {
@@ -919,9 +905,8 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
     c->shape_nz = L;
     realloc_state(c, V, E, T, false);
   } else {
-    // an earlier extraction that stopped early may have left keys and flags
+    // an earlier extraction that stopped early may have left keys
     PC_CUDA(cudaMemsetAsync(c->bufs.table, 0xff, 32 * c->Tcap, c->stream));
-    PC_CUDA(cudaMemsetAsync(c->bufs.flags, 0, sizeof(uint32_t) * 2 * (c->Ecap / 32), c->stream));
   }
   if (dom && (c->Vcap < dom->nv0 || c->Ecap < dom->ne0))
     realloc_state(c, std::max(c->Vcap, dom->nv0), std::max(c->Ecap, dom->ne0), c->Tcap, false);
@@ -1078,7 +1063,7 @@ void StateBufs::release(pc_ctx* c) {
   ctx_free(c, E);
   ctx_free(c, list0);
   ctx_free(c, list1);
-  ctx_free(c, flags);
+  ctx_free(c, nx);
   ctx_free(c, vlist);
   ctx_free(c, table);
   ctx_free(c, tape_pq);
@@ -1416,10 +1401,9 @@ constexpr size_t kNaOffZ1 = kNaOffZ0 + kNaZBytes;
 constexpr size_t kNaOffEsc = kNaOffZ1 + kNaZBytes;
 constexpr size_t kNaOffExc = kNaOffEsc + na_align(4 * kNaMaxV);
 constexpr size_t kNaOffList0 = kNaOffExc + na_align(4 * kNaMaxV);
-constexpr size_t kNaOffList1 = kNaOffList0 + na_align(16 * kNaMaxE);
-constexpr size_t kNaFlagBytes = na_align(4 * 2 * (kNaMaxE / 32));
-constexpr size_t kNaOffFlags = kNaOffList1 + na_align(16 * kNaMaxE);
-constexpr size_t kNaOffTable = kNaOffFlags + kNaFlagBytes;
+constexpr size_t kNaOffList1 = kNaOffList0 + na_align(12 * kNaMaxE);
+constexpr size_t kNaOffNx = kNaOffList1 + na_align(12 * kNaMaxE);
+constexpr size_t kNaOffTable = kNaOffNx + na_align(2 * kNaMaxE);
 constexpr size_t kNaOffCnt = kNaOffTable + na_align(32 * kNaMaxT);
 constexpr size_t kNaOffG = kNaOffCnt + na_align(sizeof(Counters) * (kNaMaxN + 1));
 constexpr size_t kNaBytes = kNaOffG + na_align(sizeof(Global));
@@ -1533,7 +1517,7 @@ extern "C" pc_status pc_extract_noalloc(int L, const int32_t* widths, const doub
     c.bufs.exc = base + kNaOffExc;
     c.bufs.list0 = base + kNaOffList0;
     c.bufs.list1 = base + kNaOffList1;
-    c.bufs.flags = base + kNaOffFlags;
+    c.bufs.nx = base + kNaOffNx;
     c.bufs.table = base + kNaOffTable;
     c.cnt = base + kNaOffCnt;
     c.g = base + kNaOffG;
@@ -1546,7 +1530,6 @@ extern "C" pc_status pc_extract_noalloc(int L, const int32_t* widths, const doub
     PC_CUDA(cudaGetLastError());
     // the scratch keeps the previous call's contents: reset what must start empty
     PC_CUDA(cudaMemsetAsync(base + kNaOffTable, 0xff, 32 * kNaMaxT, c.stream));
-    PC_CUDA(cudaMemsetAsync(base + kNaOffFlags, 0, kNaFlagBytes, c.stream));
     PC_CUDA(cudaMemsetAsync(base + kNaOffCnt, 0, sizeof(Counters) * (nn + 1), c.stream));
     net.rd_batch = rd_batch_size(mw, D, net.S);
     c.res_smem = rd_layout(net.rd_batch, mw, D, net.S).total;

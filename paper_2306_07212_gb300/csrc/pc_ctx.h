@@ -56,7 +56,7 @@ struct StateBufs {
   void* E = nullptr;
   void* list0 = nullptr;  // splitting edges of the even / odd neurons' steps
   void* list1 = nullptr;
-  void* flags = nullptr;  // two bitmaps of Ecap bits: edge in list0 / list1
+  void* nx = nullptr;     // each edge's next crossing neuron
   void* vlist = nullptr;
   void* table = nullptr;
   void* tape_pq = nullptr;

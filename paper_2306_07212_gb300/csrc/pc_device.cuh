@@ -12,10 +12,10 @@
 //   exc   [Vcap]      float32 estimate of the vertex's coordinate error
 //   SIG   [S][Vcap]   packed sign vectors, 2 bits per entry, word-major
 //   EU/EW [Ecap]      int32 edge endpoints (EW = EU + Ecap)
-//   list  [2][Ecap]   splitting edges (edge id, V+, V-) of a step, two lists
+//   list  [2][3][Ecap] splitting edges (edge id, V+, V-) of a step, two lists
 //                     by neuron parity: one is split while the next neuron's
 //                     is built
-//   flags [2][Ecap/32] bit e set iff edge e is in the list of that parity
+//   nx    [Ecap]      the next neuron of the layer that crosses the edge
 //   table [2][Tcap]   open-addressing hash tables of 2-face keys, by parity
 //   cnt   [N+1]       per-neuron counters (slot n+1 belongs to neuron n)
 #pragma once
@@ -136,8 +136,8 @@ struct State {
   uint64_t* SIG;
   int32_t* EU;
   int32_t* EW;
-  int4* list[2];         // splitting edges (edge, V+, V-, 0) of the steps of each neuron parity
-  uint32_t* flags[2];    // bit e of flags[a]: edge e is in list[a]
+  int32_t* list[2];      // splitting edges of the steps of each neuron parity: rows edge, V+, V- of Ecap
+  uint16_t* nx;          // per edge: the next crossing neuron of the layer (kNx*)
   uint64_t* table;       // two hash tables of 2 Tcap words each (neuron parity 0, 1); slots of
                          // 16 bytes (fingerprint, payload), or 8 bytes (tag | payload) inline
   int4* vlist;           // per edge: (v_a, v_b, zero ordinals, neuron + 1) of a pairing edge, else 0

@@ -7,26 +7,36 @@
 //       vertex gets its final sign: an exact zero is a genericity violation
 //       (counted, taken as +); in mixed precision a |z_j| within kappa times
 //       its FP32 error estimate is re-decided in FP64 at the exact vertex.
-//   phase_scan0    (layer start, once) step (3) for neuron 0: the edges whose
-//       endpoints have opposite signs are listed as (edge, V+, V-).
+//       The layer's sign codes go into the vertices' sign words.
+//   phase_scan0    (layer start, once) step (3) for the whole layer: the
+//       neurons that cross an edge are the entries in which its endpoints'
+//       sign words are opposite.  nx[e] = the first of them; the edges that
+//       neuron 0 crosses are listed as (edge, V+, V-).
 //   phase_step     (once per neuron, one grid-wide synchronisation each)
 //       steps (4) + (5) for the listed splitting edges of neuron i: new
 //       vertex by interpolation (FP64 t and coordinates), the edge split into
 //       E+ and E-, the parent 2-faces paired in a hash table; and, looking
-//       ahead, step (3) for neuron i + 1: the warp that splits an edge
-//       classifies its two halves and the intersecting edges it creates, the
-//       edge scan classifies every other edge.  So each step starts with its
-//       splitting edges listed and counted, and the capacity check happens
-//       before any write.
-//   phase_pack     (layer end, once) the layer's sign codes of every vertex
-//       are packed into the sign words from the signs of its values.
+//       ahead, step (3) for neuron i + 1: the warp that splits an edge finds
+//       the next crossing of its two halves (and lists those that neuron
+//       i + 1 crosses), and the edge scan lists every other edge with nx =
+//       i + 1.  So each step starts with its splitting edges listed and
+//       counted, and the capacity check happens before any write.
 //
-// During a layer the sign of a vertex w.r.t. a neuron j of the layer is the
-// sign of its stored value z_j (0 exactly on the folded hyperplane); the
-// values are made consistent with that rule when they are created, so the
-// packed codes equal what step (2) decides.  The sign words hold the earlier
-// layers' entries; a new vertex's words are written complete (earlier layers
-// from its edge's endpoints, this layer from the values) when it is created.
+// The scan of a step reads two bytes per edge.  (Reading every edge's two
+// endpoints and gathering their values instead, step after step, was 40 % of
+// the loop's time on a net of 1e7 vertices and 5e7 edges: it moved 8 bytes
+// per edge from HBM and two 32-byte sectors per edge from L2.)  The
+// intersecting edges of a step get their nx one step later (kFresh until
+// then): their endpoints' sign words are visible to every CTA only after the
+// grid-wide synchronisation; whether neuron i + 1 crosses them is known at
+// once from one sign bit in the hash payload.
+//
+// A new vertex's sign words are written complete when it is created: earlier
+// entries from its edge's endpoints, the later neurons of the layer from the
+// signs of its interpolated values.  During a layer the sign of a vertex
+// w.r.t. a neuron j of the layer is the sign of its stored value z_j (0
+// exactly on the folded hyperplane); values and codes are made consistent
+// when they are created.
 //
 // A new vertex whose value for a later neuron of the layer is within the FP32
 // filter is re-decided in FP64 by its CTA right after it is created, before
@@ -39,22 +49,31 @@
 namespace pc {
 
 constexpr int kPairCap = 1024;         // intersecting edges a CTA buffers before it appends them
-constexpr int kLaCap = 1024;           // look-ahead list entries a CTA buffers
+constexpr int kLaCap = 64;             // list entries a warp buffers
 constexpr int kPendCap = 2 * kBlock;   // vertices a CTA queues for an FP64 re-decision
+constexpr int kScanTile = 1024;        // edges a warp scans at a time (4 x 16 bytes of nx per lane)
+
+// nx[e]: the next neuron of the layer (local index) that crosses edge e, or
+constexpr uint16_t kNxNone = 0x7fff;    // no neuron left
+constexpr uint16_t kNxFresh = 0x7ffe;   // made by the last step's pairing, not known yet
+constexpr uint16_t kNxListed = 0x8000;  // in the next step's list already
+
+struct ListEntry {
+  int e, p, q;                         // splitting edge, V+, V-
+};
 
 struct Smem {
   long long pend[kPendCap];
   int4 pairs[kPairCap];                // (v_a, v_b, zero ordinals, neuron + 1)
   unsigned char pnext[kPairCap];       // bit 0: v_a is - at the next neuron, bit 1: v_b is -
-  int4 la[kLaCap];                     // split halves that split again at the next neuron
+  ListEntry la[kWarps][kLaCap];        // the warps' list entries for the next neuron
+  int lac[kWarps];
   int npairs;
   int npairla;                         // buffered pairs that split at the next neuron
-  int nla;
   int cursor;
   int npend;
-  int wcnt[kWarps];
-  int use_smem;
-  long long pbase, lbase, sbase;
+  int tile;                            // next scan tile of this CTA
+  long long pbase, lbase;
   int zlist[kWarps][16];
   float nrl[3 * kMaxWidth];            // the layer's per-neuron norms (NetDesc::nrm)
   int nrl_layer;                       // layer staged in nrl, -1: none
@@ -93,28 +112,52 @@ __device__ __forceinline__ bool step_counts(const State& st, int n, long long& n
   return nV >= 0 && nV <= st.Vcap && nE >= 0 && nE <= st.Ecap;
 }
 
-__device__ __forceinline__ void set_flag(uint32_t* f, long long e) {
-  atomicOr(f + (e >> 5), 1u << (e & 31));
+__device__ __forceinline__ void list_store(int32_t* list, long long Ecap, long long k, const ListEntry& x) {
+  list[k] = x.e;
+  list[Ecap + k] = x.p;
+  list[2 * Ecap + k] = x.q;
 }
 
-// Appends this lane's `c` (0..2) list entries with one atomic per warp; all
-// lanes must call it.
-__device__ __forceinline__ void warp_append(int c, const int4* ent, int4* list, uint32_t* flags, long long* counter) {
+// Appends the warp's buffered entries to the list with one atomic.
+__device__ __forceinline__ void warp_flush(const State& st, const ListEntry* la, int& lac, int32_t* list,
+                                           long long* counter) {
   const int lane = threadIdx.x & 31;
-  int x = c;
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  const int tot = __shfl_sync(0xffffffffu, x, 31);
-  if (tot == 0) return;
+  __syncwarp();
   long long base = 0;
-  if (lane == 31) base = atomic_add_ll(counter, (long long)tot);
-  base = __shfl_sync(0xffffffffu, base, 31) + (x - c);
-  for (int t = 0; t < c; ++t) {
-    list[base + t] = ent[t];
-    set_flag(flags, ent[t].x);
+  if (lane == 0) base = atomic_add_ll(counter, (long long)lac);
+  base = __shfl_sync(0xffffffffu, base, 0);
+  for (int t = lane; t < lac; t += 32) list_store(list, st.Ecap, base + t, la[t]);
+  __syncwarp();
+  lac = 0;
+}
+
+// One entry (hit) per lane into the warp's buffer, appended when it fills
+// (lac: entries held, warp-uniform).  All lanes call it.
+__device__ __forceinline__ void warp_list(const State& st, bool hit, const ListEntry& x, ListEntry* la, int& lac,
+                                          int32_t* list, long long* counter) {
+  const unsigned b = __ballot_sync(0xffffffffu, hit);
+  if (!b) return;
+  const int n = __popc(b);
+  if (lac + n > kLaCap) warp_flush(st, la, lac, list, counter);
+  if (hit) la[lac + __popc(b & ((1u << (threadIdx.x & 31)) - 1u))] = x;
+  lac += n;
+}
+
+// Bit 2r of the result is set iff entry 32 w + r is + in one word and - in
+// the other: neuron r separates the two vertices.
+__device__ __forceinline__ uint64_t opposite(uint64_t a, uint64_t b) {
+  return ((a & (b >> 1)) | (b & (a >> 1))) & kEvenBits;
+}
+
+// The first entry in [e_from, e_end) that separates vertices u and v (their
+// stored sign words), or -1.
+__device__ __forceinline__ int first_opposite(const State& st, long long u, long long v, int e_from, int e_end) {
+  for (int w = e_from >> 5; 32 * w < e_end; ++w) {
+    uint64_t c = opposite(st.SIG[(long long)w * st.Vcap + u], st.SIG[(long long)w * st.Vcap + v]);
+    c &= entries_below(w, e_end) & ~entries_below(w, e_from);
+    if (c) return 32 * w + (__ffsll((long long)c) - 1) / 2;
   }
+  return -1;
 }
 
 // ---------------------------------------------------------------------------
@@ -316,7 +359,10 @@ __device__ void redecide_batch(const NetDesc& net, const State& st, const long l
     Z[(long long)j * Vcap + v] = zz;
     atomic_add_ll(&st.cnt[n0 + j + 1].nfilter, 1ll);
     if (und) atomic_add_ll(&st.cnt[n0 + j + 1].nundecided, 1ll);
-    if ((z32 < 0.f) != minus) {  // the FP32 sign was wrong: how close to the filter's edge was it?
+    if ((z32 < 0.f) != minus) {  // the FP32 sign was wrong: its code 01 <-> 10; how close to the filter's edge was it?
+      const int entry = m + n0 + j;
+      atomicXor(reinterpret_cast<unsigned long long*>(st.SIG) + (long long)(entry >> 5) * Vcap + v,
+                3ull << (2 * (entry & 31)));
       atomicAdd(&st.g->flips, 1);
       atomicMax(&st.g->flip_margin_bits, __float_as_int(est > 0.f ? fabsf(z32) / est : 0.f));
     }
@@ -355,17 +401,25 @@ __device__ __noinline__ void phase_decide(const NetDesc& net, const State& st, i
   if (threadIdx.x == 0) sm.npend = 0;
   __syncthreads();
   const long long G = gridDim.x;
+  const int e0 = net.m + n0;
   for (long long round = 0; round * G * kBlock < nV; ++round) {
     const long long v = (round * G + blockIdx.x) * kBlock + threadIdx.x;
     if (v < nV) {
       bool filt = false;
       const float esc = MIXED ? st.esc[v] : 0.f;
+      // the layer's codes: 01, or 10 for a negative value
+      uint64_t word = st.SIG[(long long)(e0 >> 5) * Vcap + v] & entries_below(e0 >> 5, e0);
       for (int j = 0; j < H; ++j) {
         ZT z = Z[(long long)j * Vcap + v];
         if (z == ZT(0)) {  // on a folded hyperplane it was not created on: not generic
           z = tiny_value<ZT>();
           Z[(long long)j * Vcap + v] = z;
           atomic_add_ll(&st.cnt[n0 + j + 1].ndegenerate, 1ll);
+        }
+        word |= (z < ZT(0) ? kMinus : kPlus) << (2 * ((e0 + j) & 31));
+        if (((e0 + j) & 31) == 31 || j == H - 1) {
+          st.SIG[(long long)((e0 + j) >> 5) * Vcap + v] = word;
+          word = 0;
         }
         if (MIXED)
           filt = filt || fabsf(static_cast<float>(z)) <=
@@ -385,160 +439,132 @@ __device__ __noinline__ void phase_decide(const NetDesc& net, const State& st, i
 }
 
 // ---------------------------------------------------------------------------
-// Step (3) for one neuron over the edges [0, nE): an edge splits iff its
-// endpoints' values in zrow have opposite signs.  Edges flagged in fcur are
-// skipped (they split in the current step, whose warps classify their
-// halves); fcur is cleared on the way.  classify = false only clears.  A CTA
-// takes 2048 consecutive edges per iteration (one 128-edge tile per warp,
-// CTAs round-robin) and reserves its list entries with one atomic.
-// The flag word and the four edges (endpoint pairs) of one lane of a tile.
-struct ScanTile {
-  uint32_t fw;
-  int4 eu, ew;
-  int nvalid;
-};
-
-// nE may be the edge capacity (a load issued before the count is known):
-// scan_edges takes the valid edges from the actual count.
-__device__ __forceinline__ ScanTile scan_load(const State& st, const uint32_t* fcur, long long idx0, long long nE,
-                                              bool classify) {
-  ScanTile T;
-  T.fw = (fcur != nullptr && idx0 < nE) ? fcur[idx0 >> 5] : 0u;
-  T.eu = make_int4(0, 0, 0, 0);
-  T.ew = make_int4(0, 0, 0, 0);
-  T.nvalid = 0;
-  if (classify && idx0 < nE) {
-    T.nvalid = nE - idx0 >= 4 ? 4 : int(nE - idx0);
-    if (T.nvalid == 4) {
-      T.eu = *reinterpret_cast<const int4*>(st.EU + idx0);
-      T.ew = *reinterpret_cast<const int4*>(st.EW + idx0);
-    } else {
-      int* pu = &T.eu.x;
-      int* pw = &T.ew.x;
-      for (int q = 0; q < T.nvalid; ++q) {
-        pu[q] = st.EU[idx0 + q];
-        pw[q] = st.EW[idx0 + q];
-      }
-    }
-  }
-  return T;
+// The code of vertex v at an entry is - (it has a code there).
+__device__ __forceinline__ bool minus_at(const State& st, long long v, int entry) {
+  return ((st.SIG[(long long)(entry >> 5) * st.Vcap + v] >> (2 * (entry & 31))) & 3ull) == kMinus;
 }
 
-__device__ __forceinline__ long long scan_first_idx0() {
-  return (long long)blockIdx.x * (4ll * kBlock) + (threadIdx.x >> 5) * 128 + 4 * (threadIdx.x & 31);
-}
-
-// first: this lane's part of the CTA's first iteration (scan_load at
-// scan_first_idx0()), loaded by the caller early.  The entries go to the
-// CTA's look-ahead buffer sm.la while it has room (the caller flushes it),
-// else straight to the list with one reservation per CTA iteration.
-template <typename ZT>
-__device__ void scan_edges(const State& st, const ZT* zrow, long long nE, long long nV, uint32_t* fcur,
-                           bool classify, int4* lnext, uint32_t* fnext, long long* counter, int n, Smem& sm,
-                           const ScanTile& first) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Step (3) for neuron i + 1 (entry e + 1) during step i: lists the edges with
+// nx = i + 1 among the first nA, whose nx is known, and finds nx of the
+// others (made by the last step's pairing).  The warps of a CTA take its
+// tiles (kScanTile known edges or 32 fresh ones; tiles dealt to the CTAs
+// round-robin) until none is left, so the scan runs beside the splits.  An
+// edge that splits in this step has another nx before and after its warp
+// rewrites it, so it is never listed here.
+__device__ __forceinline__ void scan_tiles(const State& st, int i, int e, int e_end, long long nA, long long nE,
+                                           long long nV, int n, Smem& sm, ListEntry* la, int& lac, int32_t* lnext,
+                                           long long* counter) {
+  const int lane = threadIdx.x & 31;
   const long long G = gridDim.x;
-  constexpr long long kSpan = 4ll * kBlock;
-  const long long iters = (nE + kSpan * G - 1) / (kSpan * G);
-  // the next iteration's flags and endpoints are loaded while this one is classified
-  ScanTile nxt = first;
-  for (long long it = 0; it < iters; ++it) {
-    const long long idx0 = (it * G + blockIdx.x) * kSpan + warp * 128 + 4 * lane;
-    const ScanTile T = nxt;
-    if (it + 1 < iters) nxt = scan_load(st, fcur, idx0 + kSpan * G, nE, classify);
-    const int nvalid = idx0 >= nE ? 0 : (nE - idx0 >= 4 ? 4 : int(nE - idx0));
-    const uint32_t skip = (T.fw >> (idx0 & 31)) & 0xFu;
-    if (fcur != nullptr) {
-      __syncwarp();
-      if ((lane & 7) == 0 && idx0 < nE && T.fw) fcur[idx0 >> 5] = 0u;
-    }
-    if (!classify) continue;  // uniform
-    const int* pu = &T.eu.x;
-    const int* pw = &T.ew.x;
-    int4 ent[4];
-    int c = 0;
-    uint32_t nib = 0;
+  const long long TA = (nA + kScanTile - 1) / kScanTile, TB = (nE - nA + 31) / 32;
+  const uint32_t want = uint32_t(i + 1) * 0x10001u;
+  for (;;) {
+    int k = 0;
+    if (lane == 0) k = atomicAdd(&sm.tile, 1);
+    k = __shfl_sync(0xffffffffu, k, 0);
+    const long long t = (long long)k * G + blockIdx.x;
+    if (t >= TA + TB) return;
+    if (t < TA) {
+      const long long base = t * kScanTile + 8 * lane;
+      uint4 x[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (q >= nvalid || ((skip >> q) & 1u)) continue;
-      const int u = pu[q], w = pw[q];
-      if (u < 0 || u >= nV || w < 0 || w >= nV) {
-        report_corrupt(st.g, 6, n, idx0 + q, u, w);  // never index with it
-        continue;
+      for (int h = 0; h < 4; ++h)
+        x[h] = base + 256 * h < nA ? *reinterpret_cast<const uint4*>(st.nx + base + 256 * h)
+                                   : make_uint4(~0u, ~0u, ~0u, ~0u);
+      uint32_t hits = 0;  // bit 8 h + q: edge base + 256 h + q
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const uint32_t w[4] = {x[h].x, x[h].y, x[h].z, x[h].w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t m = __vcmpeq2(w[q], want);
+          if (m) hits |= ((m & 1u) | ((m >> 15) & 2u)) << (8 * h + 2 * q);
+        }
       }
-      const bool su = zrow[u] < ZT(0), sv = zrow[w] < ZT(0);
-      if (su != sv) {
-        ent[c++] = make_int4(int(idx0 + q), su ? w : u, su ? u : w, 0);
-        nib |= 1u << q;
+      while (__any_sync(0xffffffffu, hits != 0)) {
+        bool hit = false;
+        ListEntry ent{};
+        if (hits) {
+          const int bit = __ffs(hits) - 1;
+          hits &= hits - 1;
+          const long long ed = base + 256 * (bit >> 3) + (bit & 7);
+          if (ed < nA) {
+            const int u = st.EU[ed], w = st.EW[ed];
+            if (u < 0 || u >= nV || w < 0 || w >= nV) {
+              report_corrupt(st.g, 6, n, ed, u, w);  // never index with it
+            } else {
+              const bool su = minus_at(st, u, e + 1);
+              ent = ListEntry{int(ed), su ? w : u, su ? u : w};
+              hit = true;
+            }
+          }
+        }
+        warp_list(st, hit, ent, la, lac, lnext, counter);
       }
-    }
-    int x = c;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) sm.wcnt[warp] = x;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      long long tot = 0;
-      for (int w = 0; w < kWarps; ++w) {
-        const int cw = sm.wcnt[w];
-        sm.wcnt[w] = int(tot);
-        tot += cw;
+    } else {
+      const long long ed = nA + (t - TA) * 32 + lane;
+      bool hit = false;
+      ListEntry ent{};
+      if (ed < nE && *(volatile const uint16_t*)(st.nx + ed) == kNxFresh) {
+        const int u = st.EU[ed], w = st.EW[ed];
+        if (u < 0 || u >= nV || w < 0 || w >= nV) {
+          report_corrupt(st.g, 7, n, ed, u, w);
+        } else {
+          const int f = first_opposite(st, u, w, e + 1, e_end);
+          hit = f == e + 1;
+          if (hit) {
+            const bool su = minus_at(st, u, e + 1);
+            ent = ListEntry{int(ed), su ? w : u, su ? u : w};
+          }
+          st.nx[ed] = f < 0 ? kNxNone : (hit ? kNxListed : uint16_t(f - e + i));
+        }
       }
-      if (sm.nla + tot <= kLaCap) {
-        sm.use_smem = 1;
-        sm.sbase = sm.nla;
-        sm.nla += int(tot);
-      } else {
-        sm.use_smem = 0;
-        sm.sbase = atomic_add_ll(counter, tot);
-      }
+      warp_list(st, hit, ent, la, lac, lnext, counter);
     }
-    __syncthreads();
-    if (c) {
-      const long long base = sm.sbase + sm.wcnt[warp] + (x - c);
-      if (sm.use_smem) {
-        for (int t = 0; t < c; ++t) sm.la[base + t] = ent[t];  // flagged when flushed
-      } else {
-        for (int t = 0; t < c; ++t) lnext[base + t] = ent[t];
-      }
-    }
-    if (!sm.use_smem) {
-      uint32_t word = nib << (idx0 & 31);  // the 8 lanes of a flag word OR their nibbles
-      word |= __shfl_xor_sync(0xffffffffu, word, 1);
-      word |= __shfl_xor_sync(0xffffffffu, word, 2);
-      word |= __shfl_xor_sync(0xffffffffu, word, 4);
-      if ((lane & 7) == 0 && word) atomicOr(fnext + (idx0 >> 5), word);
-    }
-    __syncthreads();  // sm.use_smem / sbase are reused by the next iteration
   }
 }
 
-__device__ void flush_cta(const State& st, Counters* cur, long long* cnext, int4* lnext, uint32_t* fnext,
-                          long long ebase, bool ahead, Smem& sm);
+__device__ void flush_cta(const State& st, Counters* cur, long long* cnext, int32_t* lnext, long long ebase,
+                          bool ahead, int lac, Smem& sm);
 
-// Layer start, step (3) for neuron 0 of layer l.
-template <typename ZT>
-__device__ void phase_scan0(const NetDesc& net, const State& st, int l, Smem& sm) {
-  const int n0 = net.off[l];
+// Layer start: nx of every edge, and the list of neuron 0 of layer l.
+__device__ inline void phase_scan0(const NetDesc& net, const State& st, int l, Smem& sm) {
+  const int n0 = net.off[l], H = net.w[l + 1], e0 = net.m + n0;
   long long nV, nE;
   if (!step_counts(st, n0, nV, nE)) {
     if (threadIdx.x == 0) report_corrupt(st.g, 2, n0, nV, nE, st.Vcap);
     return;
   }
-  const ZT* zrow = static_cast<const ZT*>(st.Z[l]);
+  const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     sm.npairs = 0;
     sm.npairla = 0;
-    sm.nla = 0;
   }
-  __syncthreads();
-  const ScanTile first = scan_load(st, nullptr, scan_first_idx0(), nE, true);
-  scan_edges<ZT>(st, zrow, nE, nV, nullptr, true, st.list[n0 & 1], st.flags[n0 & 1], &st.cnt[n0 + 1].nsplit, n0, sm,
-                 first);
-  __syncthreads();
-  if (sm.nla) flush_cta(st, nullptr, &st.cnt[n0 + 1].nsplit, st.list[n0 & 1], st.flags[n0 & 1], 0, true, sm);
+  int32_t* list = st.list[n0 & 1];
+  long long* counter = &st.cnt[n0 + 1].nsplit;
+  int lac = 0;
+  const long long step = (long long)gridDim.x * kBlock;
+  for (long long base = (long long)blockIdx.x * kBlock; base < nE; base += step) {
+    const long long ed = base + threadIdx.x;
+    bool hit = false;
+    ListEntry ent{};
+    if (ed < nE) {
+      const int u = st.EU[ed], w = st.EW[ed];
+      if (u < 0 || u >= nV || w < 0 || w >= nV) {
+        report_corrupt(st.g, 6, n0, ed, u, w);
+      } else {
+        const int f = first_opposite(st, u, w, e0, e0 + H);
+        hit = f == e0;
+        if (hit) {
+          const bool su = minus_at(st, u, e0);
+          ent = ListEntry{int(ed), su ? w : u, su ? u : w};
+        }
+        st.nx[ed] = f < 0 ? kNxNone : (hit ? kNxListed : uint16_t(f - e0));
+      }
+    }
+    warp_list(st, hit, ent, sm.la[warp], lac, list, counter);
+  }
+  flush_cta(st, nullptr, counter, list, 0, true, lac, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -557,7 +583,7 @@ __device__ __forceinline__ bool warp_face_matches(const State& st, long long k2,
   const long long v2 = nV + k2;
   uint64_t w2 = 0, zm = 0;
   if (lane < S) {
-    w2 = __ldcg(st.SIG + (long long)lane * st.Vcap + v2);
+    w2 = __ldcg(st.SIG + (long long)lane * st.Vcap + v2) & entries_below(lane, e);
     zm = zero_mask(w2, lane, e);
   }
   const int c = __popcll(zm);
@@ -586,40 +612,53 @@ __device__ __forceinline__ bool warp_face_matches(const State& st, long long k2,
 
 // ---------------------------------------------------------------------------
 // Appends the CTA's buffered intersecting edges (and those of them that split
-// at the next neuron) and buffered look-ahead entries: one atomic each for
-// the CTA.  All threads call it after a __syncthreads.
-__device__ void flush_cta(const State& st, Counters* cur, long long* cnext, int4* lnext, uint32_t* fnext,
-                          long long ebase, bool ahead, Smem& sm) {
-  const int np = sm.npairs, nla = sm.nla, npla = sm.npairla;
+// at the next neuron) and the warps' buffered list entries (lac of this
+// warp's): one atomic each for the CTA.  All threads call it.
+__device__ void flush_cta(const State& st, Counters* cur, long long* cnext, int32_t* lnext, long long ebase,
+                          bool ahead, int lac, Smem& sm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) sm.lac[warp] = lac;
+  __syncthreads();
+  const int np = sm.npairs, npla = sm.npairla;
+  int first = 0, nla = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    const int x = sm.lac[w];
+    if (w < warp) first += x;
+    nla += x;
+  }
+  if (np + nla == 0) return;  // uniform
   if (threadIdx.x == 0) {
-    sm.pbase = np ? atomic_add_ll(&cur->npairs, (long long)np) : 0;
-    sm.lbase = (ahead && nla + npla) ? atomic_add_ll(cnext, (long long)(nla + npla)) : 0;
+    // both positions in flight at once
+    long long pb = 0, lb = 0;
+    if (np) pb = atomic_add_ll(&cur->npairs, (long long)np);
+    if (ahead && nla + npla) lb = atomic_add_ll(cnext, (long long)(nla + npla));
+    sm.pbase = pb;
+    sm.lbase = lb;
     sm.cursor = 0;
   }
   __syncthreads();
-  const long long pb = ebase + sm.pbase;
+  const long long pb = ebase + sm.pbase, lb = sm.lbase;
   for (int t = threadIdx.x; t < np; t += kBlock) {
     const int4 rec = sm.pairs[t];
     st.EU[pb + t] = rec.x;
     st.EW[pb + t] = rec.y;
     if (st.deferred) st.vlist[pb + t] = rec;
+    if (!ahead) continue;
     const unsigned char nx = sm.pnext[t];
-    if (ahead && ((nx ^ (nx >> 1)) & 1)) {  // the new edge splits at the next neuron
+    const bool hit = (nx ^ (nx >> 1)) & 1;  // the new edge splits at the next neuron
+    st.nx[pb + t] = hit ? kNxListed : kNxFresh;
+    if (hit) {
       const int j = atomicAdd(&sm.cursor, 1);
-      lnext[sm.lbase + nla + j] = (nx & 1) ? make_int4(int(pb + t), rec.y, rec.x, 0)
-                                           : make_int4(int(pb + t), rec.x, rec.y, 0);
-      set_flag(fnext, pb + t);
+      list_store(lnext, st.Ecap, lb + nla + j,
+                 (nx & 1) ? ListEntry{int(pb + t), rec.y, rec.x} : ListEntry{int(pb + t), rec.x, rec.y});
     }
   }
-  for (int t = threadIdx.x; t < nla; t += kBlock) {
-    const int4 ent = sm.la[t];
-    lnext[sm.lbase + t] = ent;
-    set_flag(fnext, ent.x);
-  }
+  if (ahead)
+    for (int t = lane; t < lac; t += 32) list_store(lnext, st.Ecap, lb + first + t, sm.la[warp][t]);
   __syncthreads();
   if (threadIdx.x == 0) {
     sm.npairs = 0;
-    sm.nla = 0;
     sm.npairla = 0;
   }
   __syncthreads();
@@ -636,10 +675,11 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
   const bool ahead = i + 1 < H;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long G = gridDim.x;
-  const int4* lcur = st.list[n & 1];
+  const int32_t* lcur = st.list[n & 1];
   // this warp's first splitting edge, loaded together with the counters
   const long long k_first = (long long)warp * G + blockIdx.x;
-  const int4 sg_first = k_first < st.Ecap ? lcur[k_first] : make_int4(-1, -1, -1, 0);
+  ListEntry sg_next{-1, -1, -1};
+  if (k_first < st.Ecap) sg_next = ListEntry{lcur[k_first], lcur[st.Ecap + k_first], lcur[2 * st.Ecap + k_first]};
   Counters* cur = st.cnt + n + 1;
   long long nV, nE;
   if (!step_counts(st, n, nV, nE)) {
@@ -682,8 +722,8 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
   if (threadIdx.x == 0) {
     sm.npairs = 0;
     sm.npairla = 0;
-    sm.nla = 0;
     sm.npend = 0;
+    sm.tile = 0;
     sm.acc[0] = sm.acc[1] = 0;
   }
   if (sm.nrl_layer != l) {  // uniform: set by the previous step of this launch, or -1
@@ -701,8 +741,13 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
   ZT* Z = static_cast<ZT*>(st.Z[l]);
   const int e = m + n;
   const int e0 = m + net.off[l];
-  int4* lnext = st.list[(n + 1) & 1];
-  uint32_t* fnext = st.flags[(n + 1) & 1];
+  const int e_end = e0 + H;
+  // edges whose nx is known: all but those of the last step's pairing
+  const long long nA = i > 0 ? st.cnt[n].nE_before + st.cnt[n].nsplit : nE;
+  int32_t* lnext = st.list[(n + 1) & 1];
+  ListEntry* la = sm.la[warp];
+  int lac = 0;
+  bool scan = ahead;
   long long* cnext = ahead ? &st.cnt[n + 2].nsplit : nullptr;
   uint64_t* table = st.table + (long long)(n & 1) * 2 * st.Tcap;
   const long long tmask = tneed - 1;
@@ -713,11 +758,11 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
   unsigned long long paired_seen = 0;  // paired flags found by this lane's second arrivals
   const long long Wt = G * kWarps;
   const long long rounds = (total + Wt - 1) / Wt;
-  int4 sg_next = sg_first;
   for (long long rd = 0; rd < rounds; ++rd) {
     const long long k = rd * Wt + k_first;  // splits dealt over the CTAs first
-    const int4 sg_this = sg_next;
-    if (k + Wt < total) sg_next = lcur[k + Wt];  // the next round's, loaded during this one
+    const ListEntry sg = sg_next;
+    if (k + Wt < total)  // the next round's, loaded during this one
+      sg_next = ListEntry{lcur[k + Wt], lcur[st.Ecap + k + Wt], lcur[2 * st.Ecap + k + Wt]};
     // The round's new vertices are numbered CTA by CTA: CTA b holds entries
     // w G + b of the round (w < n_b = rq + [b < rr]) and gives them the
     // consecutive offsets b rq + min(b, rr) + w, a bijection onto the
@@ -730,13 +775,11 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
     bool okA = false, pend = false, bad = false;
     int32_t ed = 0, p = 0, q = 0;
     const int32_t v0 = int32_t(nV + voff);
-    uint64_t s0 = 0, zm = 0;
-    ZT zpn = ZT(0), zqn = ZT(0), z0n = ZT(0);  // values at neuron i + 1
+    uint64_t s0 = 0, sp = 0, sq = 0;  // sign words of the new vertex and its parents (lane w: word w)
     if (k < total) {
-      const int4 sg = sg_this;
-      ed = sg.x;
-      p = sg.y;  // V+
-      q = sg.z;  // V-
+      ed = sg.e;
+      p = sg.p;  // V+
+      q = sg.q;  // V-
       okA = !(ed < 0 || ed >= nE || p < 0 || p >= nV || q < 0 || q >= nV);  // warp-uniform
       if (!okA && lane == 0) report_corrupt(st.g, 4, n, ed, p, q);
     }
@@ -748,7 +791,6 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
         xp = st.X[(long long)lane * Vcap + p];
         xq = st.X[(long long)lane * Vcap + q];
       }
-      uint64_t sp = 0, sq = 0;
       if (lane < S) {
         sp = st.SIG[(long long)lane * Vcap + p];
         sq = st.SIG[(long long)lane * Vcap + q];
@@ -786,8 +828,7 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
       const ZT tz = static_cast<ZT>(t);
       // earlier layers' entries: the join of the endpoints' words
       const uint64_t below = lane < S ? entries_below(lane, e0) : 0ull;
-      const uint64_t conf = ((sp & kEvenBits) & ((sq >> 1) & kEvenBits)) | ((sq & kEvenBits) & ((sp >> 1) & kEvenBits));
-      if (conf & below) err_w |= kErrConflict;
+      if (opposite(sp, sq) & below) err_w |= kErrConflict;
       s0 = (sp | sq) & below;
       float amax = 0.f;
       float zk[2] = {0.f, 0.f};  // this lane's new values of rows lane, lane + 32 (filter)
@@ -817,6 +858,8 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
                 zj = tiny_value<ZT>();
                 atomic_add_ll(&st.cnt[net.off[l] + j + 1].ndegenerate, 1ll);
               }
+              mi = zj < ZT(0);
+              pl = !mi;
             }
             Z[(long long)j * Vcap + v0] = zj;  // row i: exactly 0
             if (TRACK) amax = fmaxf(amax, fabsf(static_cast<float>(zj)) * nrl[3 * j + 2]);
@@ -824,12 +867,6 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
           if (c == 0) zk[hh] = static_cast<float>(zj);
           plus2[hh] = __ballot_sync(0xffffffffu, pl);
           minus2[hh] = __ballot_sync(0xffffffffu, mi);
-          if (ahead && 64 * c + 32 * hh <= i + 1 && i + 1 < 64 * c + 32 * hh + 32) {  // warp-uniform
-            const int src = (i + 1) & 31;
-            zpn = __shfl_sync(0xffffffffu, zp, src);
-            zqn = __shfl_sync(0xffffffffu, zq, src);
-            z0n = __shfl_sync(0xffffffffu, zj, src);
-          }
         }
         // this chunk's codes (entries e0 + 64c ...) into the lane's word
 #pragma unroll
@@ -874,7 +911,6 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
       }
       if (lane < S) {
         st.SIG[(long long)lane * Vcap + v0] = s0;
-        zm = zero_mask(s0, lane, e);
       }
       if (lane == 0) {
         st.EU[ed] = p;
@@ -890,14 +926,39 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
         if (pend) sm.pend[atomicAdd(&sm.npend, 1)] = v0;
       }
     }
+    if (scan && !okA) {  // a warp without a split: the scan, beside the others' splits
+      scan_tiles(st, i, e, e_end, nA, nE, nV, n, sm, la, lac, lnext, cnext);
+      scan = false;
+    }
     if (MIXED) {  // FP64 re-decisions of this round's new vertices (uniform per CTA)
       __syncthreads();
       if (sm.npend > 0) drain_pending<ZT>(net, st, l, e + 1, i + 1, mw, ws, sm);
     }
     if (okA) {
       // ---- part B: the parent 2-faces (step (5)) and the look-ahead ----
-      if (ahead && pend) z0n = Z[(long long)(i + 1) * Vcap + v0];  // re-decided by this CTA
-      const bool m0n = z0n < ZT(0);
+      if (MIXED && pend && lane < S) s0 = __ldcg(st.SIG + (long long)lane * Vcap + v0);  // re-decided by this CTA
+      // the sign at the next neuron, and the next crossings of the two halves
+      const bool m0n = ahead && ((__shfl_sync(0xffffffffu, s0, (e + 1) >> 5) >> (2 * ((e + 1) & 31))) & 3ull) == kMinus;
+      if (ahead) {
+        const uint64_t later = lane < S ? entries_below(lane, e_end) & ~entries_below(lane, e + 1) : 0ull;
+        const uint64_t xp = opposite(sp, s0) & later, xq = opposite(sq, s0) & later;
+        const unsigned bp = __ballot_sync(0xffffffffu, xp != 0), bq = __ballot_sync(0xffffffffu, xq != 0);
+        const int fp = 32 * lane + (__ffsll((long long)xp) - 1) / 2, fq = 32 * lane + (__ffsll((long long)xq) - 1) / 2;
+        const int jp = bp ? __shfl_sync(0xffffffffu, fp, __ffs(bp) - 1) - e0 : kNxNone;
+        const int jq = bq ? __shfl_sync(0xffffffffu, fq, __ffs(bq) - 1) - e0 : kNxNone;
+        // E+ = (p, v0) keeps the edge's id, E- = (q, v0) is nE + k
+        const bool hp = jp == i + 1, hq = jq == i + 1;
+        if (lane == 0) {
+          st.nx[ed] = hp ? kNxListed : uint16_t(jp);
+          st.nx[nE + k] = hq ? kNxListed : uint16_t(jq);
+        }
+        const ListEntry x = lane == 0 ? (m0n ? ListEntry{ed, p, v0} : ListEntry{ed, v0, p})
+                                      : (m0n ? ListEntry{int(nE + k), q, v0} : ListEntry{int(nE + k), v0, q});
+        warp_list(st, lane == 0 ? hp : (lane == 1 && hq), x, la, lac, lnext, cnext);
+      }
+      // the 2-faces are named by the entries before this neuron
+      s0 = lane < S ? s0 & entries_below(lane, e) : 0ull;
+      const uint64_t zm = lane < S ? zero_mask(s0, lane, e) : 0ull;
       const int c0 = __popcll(zm);
       int x = c0;
       for (int o = 1; o < 32; o <<= 1) {
@@ -1034,24 +1095,14 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
           }
         }
       }
-      // look-ahead: the two halves of the split edge at neuron i + 1
-      if (ahead && lane == 0) {
-        const bool mp = zpn < ZT(0), mq = zqn < ZT(0);
-        int4 ent[2];
-        int c = 0;
-        if (mp != m0n) ent[c++] = mp ? make_int4(ed, v0, p, 0) : make_int4(ed, p, v0, 0);
-        if (mq != m0n) ent[c++] = mq ? make_int4(int(nE + k), v0, q, 0) : make_int4(int(nE + k), q, v0, 0);
-        if (c) {
-          const int b2 = atomicAdd(&sm.nla, c);  // < kLaCap: flushed every round
-          for (int t2 = 0; t2 < c; ++t2) sm.la[b2 + t2] = ent[t2];
-        }
-      }
       __syncwarp();
     }
     // keep the CTA's buffers from filling up in the next round
     __syncthreads();
-    if (sm.npairs > kPairCap - kWarps * R || sm.nla > kLaCap - 2 * kWarps)
-      flush_cta(st, cur, cnext, lnext, fnext, nE + total, ahead, sm);
+    if (sm.npairs > kPairCap - kWarps * R) {
+      flush_cta(st, cur, cnext, lnext, nE + total, ahead, lac, sm);
+      lac = 0;
+    }
   }
   if (paired_seen & kPaired64) err_w |= kErrPairing;  // a third arrival at a 2-face
   err_w = __reduce_or_sync(0xffffffffu, err_w);
@@ -1060,48 +1111,13 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
     if (ndeg_w) atomicAdd(reinterpret_cast<unsigned long long*>(&sm.acc[1]), (unsigned long long)ndeg_w);
     if (err_w) atomicOr(&st.g->error, err_w);
   }
-  __syncthreads();
+  if (scan) scan_tiles(st, i, e, e_end, nA, nE, nV, n, sm, la, lac, lnext, cnext);
+  flush_cta(st, cur, cnext, lnext, nE + total, ahead, lac, sm);
   if (threadIdx.x == 0) {
     if (sm.acc[0]) atomic_add_ll(&cur->nkeys, sm.acc[0]);
     if (sm.acc[1]) atomic_add_ll(&cur->ndegenerate, sm.acc[1]);
   }
-  // step (3) for the next neuron over the edges that did not split here
-  const ZT* znext = Z + (long long)(ahead ? i + 1 : 0) * Vcap;
-  const ScanTile scan_first = scan_load(st, st.flags[n & 1], scan_first_idx0(), nE, ahead);
-  scan_edges<ZT>(st, znext, nE, nV, st.flags[n & 1], ahead, lnext, fnext, cnext, n, sm, scan_first);
-  __syncthreads();
-  if (sm.npairs || sm.nla) flush_cta(st, cur, cnext, lnext, fnext, nE + total, ahead, sm);
   return false;
-}
-
-// ---------------------------------------------------------------------------
-// Layer end: the codes of the layer's entries of every vertex from the signs
-// of its values (+ / - / 0 exactly on the folded hyperplane).
-template <typename ZT>
-__device__ __noinline__ void phase_pack(const NetDesc& net, const State& st, int l) {
-  const int H = net.w[l + 1];
-  const Counters* last = st.cnt + net.off[l] + H;
-  const long long nV = last->nV_before + last->nsplit;
-  if (nV < 0 || nV > st.Vcap) {
-    if (threadIdx.x == 0) report_corrupt(st.g, 12, l, nV, st.Vcap, 0);
-    return;
-  }
-  const long long Vcap = st.Vcap;
-  const ZT* Z = static_cast<const ZT*>(st.Z[l]);
-  const int e0 = net.m + net.off[l], wf = e0 >> 5, wl = (e0 + H - 1) >> 5;
-  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < nV; v += (long long)gridDim.x * blockDim.x) {
-    for (int w = wf; w <= wl; ++w) {
-      uint64_t word = w == wf ? (st.SIG[(long long)w * Vcap + v] & entries_below(w, e0)) : 0ull;
-      const int jb = 32 * w - e0 > 0 ? 32 * w - e0 : 0;
-      const int je = 32 * w + 32 - e0 < H ? 32 * w + 32 - e0 : H;
-      for (int j = jb; j < je; ++j) {
-        const ZT z = Z[(long long)j * Vcap + v];
-        const uint64_t code = z > ZT(0) ? kPlus : (z < ZT(0) ? kMinus : 0ull);
-        word |= code << (2 * ((e0 + j) & 31));
-      }
-      st.SIG[(long long)w * Vcap + v] = word;
-    }
-  }
 }
 
 }  // namespace pc
