@@ -27,6 +27,9 @@
 
 namespace pc {
 
+constexpr int kAdjLd = 33;  // row stride of the staged tiles of 32 vertices
+constexpr int kAdjSmemMax = sizeof(float) * 2 * kMaxWidth * kAdjLd;
+
 __global__ void k_adj_init(const double* gx, float* xbar, long long nV, long long Vcap, int D) {
   const long long n = nV * D;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
@@ -59,22 +62,23 @@ __global__ void k_adj_split(NetDesc net, State st, float* xbar, float* zbar, int
         tb += xb * static_cast<float>(st.X[(long long)lane * Vcap + q] - st.X[(long long)lane * Vcap + p]);
       }
     }
+    const ZT* zp = Z + (long long)p * H;
+    const ZT* zq = Z + (long long)q * H;
     for (int j = lane; j < H; j += 32) {
       if (j == i) continue;
-      const float zb = zbar[(long long)j * Vcap + v0];
+      const float zb = zbar[v0 * H + j];
       if (zb == 0.f) continue;
-      atomicAdd(&zbar[(long long)j * Vcap + p], (1.f - tf) * zb);
-      atomicAdd(&zbar[(long long)j * Vcap + q], tf * zb);
-      tb += zb * static_cast<float>(static_cast<double>(Z[(long long)j * Vcap + q]) -
-                                    static_cast<double>(Z[(long long)j * Vcap + p]));
+      atomicAdd(&zbar[(long long)p * H + j], (1.f - tf) * zb);
+      atomicAdd(&zbar[(long long)q * H + j], tf * zb);
+      tb += zb * static_cast<float>(static_cast<double>(zq[j]) - static_cast<double>(zp[j]));
     }
     for (int o = 16; o > 0; o >>= 1) tb += __shfl_xor_sync(0xffffffffu, tb, o);
     if (lane == 0 && tb != 0.f) {
-      const double a = static_cast<double>(Z[(long long)i * Vcap + p]);
-      const double b = static_cast<double>(Z[(long long)i * Vcap + q]);
+      const double a = static_cast<double>(zp[i]);
+      const double b = static_cast<double>(zq[i]);
       const double d2 = (a - b) * (a - b);
-      atomicAdd(&zbar[(long long)i * Vcap + p], static_cast<float>(tb * (-b) / d2));
-      atomicAdd(&zbar[(long long)i * Vcap + q], static_cast<float>(tb * a / d2));
+      atomicAdd(&zbar[(long long)p * H + i], static_cast<float>(tb * (-b) / d2));
+      atomicAdd(&zbar[(long long)q * H + i], static_cast<float>(tb * a / d2));
     }
   }
 }
@@ -87,38 +91,34 @@ template <typename ZT>
 __global__ void __launch_bounds__(512) k_adj_wgrad(NetDesc net, State st, const float* zbar, double* gW, int l,
                                                    long long nVl) {
   extern __shared__ float sh[];
-  constexpr int EPT = 32, TV = 32;
+  constexpr int EPT = 32, TV = 32, LD = kAdjLd;  // rows padded: a tile is stored vertex by vertex, read row by row
   const int H = net.w[l + 1], K = net.w[l];
-  float* zt = sh;            // [H][TV]
-  float* at = sh + H * TV;   // [K][TV]
+  float* zt = sh;            // [H][LD]
+  float* at = sh + H * LD;   // [K][LD]
   const long long Vcap = st.Vcap;
   const ZT* Zin = static_cast<const ZT*>(st.Z[l > 0 ? l - 1 : 0]);
-  const int ebase = net.m + (l > 0 ? net.off[l - 1] : 0);
   const int e0 = blockIdx.y * blockDim.x * EPT;
   float acc[EPT];
 #pragma unroll
   for (int q = 0; q < EPT; ++q) acc[q] = 0.f;
   float bacc = 0.f;
   for (long long base = (long long)blockIdx.x * TV; base < nVl; base += (long long)gridDim.x * TV) {
-    for (int t = threadIdx.x; t < (H + K) * TV; t += blockDim.x) {
-      const int r = t / TV, c = t % TV;
-      const long long v = base + c;
+    for (int t = threadIdx.x; t < H * TV; t += blockDim.x) {
+      const int c = t / H, r = t - c * H;
+      zt[r * LD + c] = base + c < nVl ? zbar[base * H + t] : 0.f;
+    }
+    for (int t = threadIdx.x; t < K * TV; t += blockDim.x) {
+      const int c = t / K, k = t - c * K;
       float val = 0.f;
-      if (v < nVl) {
-        if (r < H) {
-          val = zbar[(long long)r * Vcap + v];
+      if (base + c < nVl) {
+        if (l == 0) {
+          val = static_cast<float>(st.X[(long long)k * Vcap + base + c]);
         } else {
-          const int k = r - H;
-          if (l == 0) {
-            val = static_cast<float>(st.X[(long long)k * Vcap + v]);
-          } else {
-            const int entry = ebase + k;
-            const bool act = ((st.SIG[(long long)(entry >> 5) * Vcap + v] >> (2 * (entry & 31))) & 3ull) == kPlus;
-            val = act ? static_cast<float>(Zin[(long long)k * Vcap + v]) : 0.f;
-          }
+          const ZT z = Zin[base * K + t];
+          val = z > ZT(0) ? static_cast<float>(z) : 0.f;  // active iff its sign entry is +
         }
       }
-      sh[r * TV + c] = val;
+      at[k * LD + c] = val;
     }
     __syncthreads();
 #pragma unroll
@@ -128,12 +128,12 @@ __global__ void __launch_bounds__(512) k_adj_wgrad(NetDesc net, State st, const 
         const int j = e / K, k = e % K;
         float s = 0.f;
 #pragma unroll 8
-        for (int c = 0; c < TV; ++c) s = fmaf(zt[j * TV + c], at[k * TV + c], s);
+        for (int c = 0; c < TV; ++c) s = fmaf(zt[j * LD + c], at[k * LD + c], s);
         acc[q] += s;
       }
     }
     if (blockIdx.y == 0 && threadIdx.x < H)
-      for (int c = 0; c < TV; ++c) bacc += zt[threadIdx.x * TV + c];
+      for (int c = 0; c < TV; ++c) bacc += zt[threadIdx.x * LD + c];
     __syncthreads();
   }
 #pragma unroll
@@ -144,19 +144,23 @@ __global__ void __launch_bounds__(512) k_adj_wgrad(NetDesc net, State st, const 
   if (blockIdx.y == 0 && threadIdx.x < H && bacc != 0.f) atomicAdd(&gW[net.bofs[l] + threadIdx.x], (double)bacc);
 }
 
-// Layer start, value part: zbar_{l-1}[k][v] = act'_k(v) sum_j W_l[j][k] zbar_l[j][v].
+// Layer start, value part: zbar_{l-1}[v][k] = act'_k(v) sum_j W_l[j][k] zbar_l[v][j].
+// Consecutive threads take consecutive k, so weights and rows are coalesced
+// and zbar_l[v][j] is one broadcast.
+template <typename ZT>
 __global__ void k_adj_back(NetDesc net, State st, const float* zbar, float* zprev, int l, long long nVl) {
   const int H = net.w[l + 1], K = net.w[l];
-  const long long Vcap = st.Vcap;
   const float* W = net.W32 + net.wofs[l];
-  const int k = blockIdx.y;
-  const int entry = net.m + net.off[l - 1] + k;
-  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < nVl; v += (long long)gridDim.x * blockDim.x) {
-    const bool act = ((st.SIG[(long long)(entry >> 5) * Vcap + v] >> (2 * (entry & 31))) & 3ull) == kPlus;
+  const ZT* Zin = static_cast<const ZT*>(st.Z[l - 1]);
+  const long long total = nVl * K;
+  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
+    const long long v = t / K;
+    const int k = int(t - v * K);
+    const float* zb = zbar + v * H;
     float s = 0.f;
-    if (act)
-      for (int j = 0; j < H; ++j) s = fmaf(W[(long long)j * K + k], zbar[(long long)j * Vcap + v], s);
-    zprev[(long long)k * Vcap + v] = s;
+    if (Zin[t] > ZT(0))  // active iff its sign entry is +
+      for (int j = 0; j < H; ++j) s = fmaf(W[(long long)j * K + k], zb[j], s);
+    zprev[t] = s;
   }
 }
 
@@ -178,17 +182,16 @@ static void run_backward(pc_ctx* c, const State& st, float* xbar, float* zb[2], 
     const long long nVl = s0.nV_before + s0.nsplit;
     const int H = net.w[l + 1], K = net.w[l];
     const int gy = (H * K + 512 * 32 - 1) / (512 * 32);
-    const size_t smem = sizeof(float) * (H + K) * 32;  // <= kAdjSmemMax (widths <= 256)
+    const size_t smem = sizeof(float) * (H + K) * kAdjLd;  // <= kAdjSmemMax (widths <= 256)
     const int gx = int(std::max<long long>(1, std::min<long long>((nVl + 31) / 32, 2 * c->num_sms)));
     k_adj_wgrad<ZT><<<dim3(gx, gy), 512, smem, c->stream>>>(net, st, zl, gW, l, nVl);
     if (l > 0) {
-      const int gb = int(std::max<long long>(1, std::min<long long>((nVl + 255) / 256, 4 * c->num_sms)));
-      k_adj_back<<<dim3(gb, K), 256, 0, c->stream>>>(net, st, zl, zb[(l - 1) & 1], l, nVl);
+      const int gb = int(std::max<long long>(1, std::min<long long>((nVl * K + 255) / 256, 16 * c->num_sms)));
+      k_adj_back<ZT><<<gb, 256, 0, c->stream>>>(net, st, zl, zb[(l - 1) & 1], l, nVl);
     }
   }
 }
 
-constexpr int kAdjSmemMax = sizeof(float) * 2 * kMaxWidth * 32;
 
 }  // namespace pc
 

@@ -352,6 +352,15 @@ __global__ void k_store_rows(const T* src, long long n, int rows, T* dst, long l
   }
 }
 
+// The values' rows: dst[i][j] = src[perm[i]][j], j < H.
+template <typename T>
+__global__ void k_gather_items(const T* src, const int* perm, long long n, int H, T* dst) {
+  const long long total = n * H;
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < total;
+       k += (long long)gridDim.x * blockDim.x)
+    dst[k] = src[(long long)perm[k / H] * H + k % H];
+}
+
 // Edges renumbered to the vertex ranks, counted per smaller endpoint.
 __global__ void k_edge_count(int32_t* EU, int32_t* EW, const int* rank, long long nE, int* count) {
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nE; e += (long long)gridDim.x * blockDim.x) {
@@ -558,7 +567,14 @@ void pc_canonicalize(pc_ctx* c) {
   };
   permute(c->bufs.X, 8, c->net.D);
   permute(c->bufs.SIG, 8, c->net.S);
-  permute(pc_make_state(c).Z[c->net.L - 1], zs, H);
+  void* Z = pc_make_state(c).Z[c->net.L - 1];
+  if (zs == 8)
+    k_gather_items<uint64_t><<<grid_for(nV * H), 256, 0, s>>>(static_cast<const uint64_t*>(Z), P, nV, H,
+                                                             static_cast<uint64_t*>(work));
+  else
+    k_gather_items<uint32_t><<<grid_for(nV * H), 256, 0, s>>>(static_cast<const uint32_t*>(Z), P, nV, H,
+                                                             static_cast<uint32_t*>(work));
+  check(cudaMemcpyAsync(Z, work, zs * H * nV, cudaMemcpyDeviceToDevice, s));
   if (c->net.precision != PC_PREC_FP64) {
     permute(c->bufs.esc, 4, 1);
     permute(c->bufs.exc, 4, 1);

@@ -208,7 +208,6 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
   const long long Vcap = st.Vcap;
   ZT* Zout = static_cast<ZT*>(st.Z[l]);
   const ZT* Zin = static_cast<const ZT*>(st.Z[l > 0 ? l - 1 : 0]);
-  const int ebase = net.m + (l > 0 ? net.off[l - 1] : 0);
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < nV;
        v += (long long)gridDim.x * blockDim.x) {
     ZT acc[TJ];
@@ -228,16 +227,9 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
     } else {
 #pragma unroll
       for (int jj = 0; jj < TJ; ++jj) acc[jj] = bs[jj];
-      uint64_t word = 0;
-      int cw = -1;
       for (int kk = 0; kk < K; ++kk) {
-        const int entry = ebase + kk, wi = entry >> 5;
-        if (wi != cw) {
-          word = st.SIG[(long long)wi * Vcap + v];
-          cw = wi;
-        }
-        const bool act = ((word >> (2 * (entry & 31))) & 3ull) == kPlus;
-        const ZT a = act ? Zin[(long long)kk * Vcap + v] : ZT(0);
+        const ZT z = Zin[v * K + kk];
+        const ZT a = z > ZT(0) ? z : ZT(0);  // active iff its sign entry is +, iff its value is positive
         a2 = fmaf(static_cast<float>(a), static_cast<float>(a), a2);
 #pragma unroll
         for (int jj = 0; jj < TJ; ++jj) acc[jj] = fma(Ws[jj][kk], a, acc[jj]);
@@ -245,7 +237,7 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
     }
 #pragma unroll
     for (int jj = 0; jj < TJ; ++jj)
-      if (j0 + jj < H) Zout[(long long)(j0 + jj) * Vcap + v] = acc[jj];
+      if (j0 + jj < H) Zout[v * H + j0 + jj] = acc[jj];
     if (TRACK && blockIdx.y == 0) {
       // rho_l: u/2 ||a||_2 (rounding: the running sums are bounded by
       // ||W_j||_2 ||a||_2) and the largest input error of the previous layer
@@ -263,55 +255,56 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
 // ---------------------------------------------------------------------------
 // Neuron phases: stepwise kernels and the persistent per-layer kernel.
 
+// Dynamic shared memory of these kernels: Smem, then the re-decision batch's
+// workspace (mixed precision).
+constexpr int kSmemBytes = (int)((sizeof(Smem) + 15) / 16 * 16);
+
 template <typename ZT, bool MIXED>
-__global__ void __launch_bounds__(kBlock, 2) k_decide(NetDesc net, State st, int l, int mw) {
-  extern __shared__ double dsm[];
-  __shared__ Smem sm;
+__global__ void __launch_bounds__(kBlock, 1) k_decide(NetDesc net, State st, int l, int mw) {
+  extern __shared__ __align__(16) unsigned char dsm[];
   if (cta_stopped(st)) return;
-  phase_decide<ZT, MIXED>(net, st, l, sm, dsm, mw);
+  phase_decide<ZT, MIXED>(net, st, l, *reinterpret_cast<Smem*>(dsm), reinterpret_cast<double*>(dsm + kSmemBytes), mw);
 }
 
 __global__ void __launch_bounds__(kBlock) k_scan0(NetDesc net, State st, int l) {
-  __shared__ Smem sm;
+  extern __shared__ __align__(16) unsigned char dsm[];
   if (cta_stopped(st)) return;
-  phase_scan0(net, st, l, sm);
+  phase_scan0(net, st, l, *reinterpret_cast<Smem*>(dsm));
 }
 
-template <typename ZT, bool MIXED>
-__global__ void __launch_bounds__(kBlock, 2) k_step(NetDesc net, State st, int l, int i, int mw) {
-  extern __shared__ double dsm[];
-  __shared__ Smem sm;
+template <typename ZT, bool MIXED, int WORDS>
+__global__ void __launch_bounds__(kBlock, 1) k_step(NetDesc net, State st, int l, int i, int mw) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  Smem& sm = *reinterpret_cast<Smem*>(dsm);
   if (cta_stopped(st)) return;
   if (threadIdx.x == 0) sm.nrl_layer = -1;
   __syncthreads();
-  phase_step<ZT, MIXED>(net, st, l, i, sm, dsm, mw);
+  phase_step<ZT, MIXED, WORDS>(net, st, l, i, sm, reinterpret_cast<double*>(dsm + kSmemBytes), mw);
 }
 
 // The neuron loop of layer l in one cooperative launch: the layer-start
 // decisions and first edge scan (prologue = 1; a launch that resumes after a
 // capacity halt skips them) and one grid barrier per neuron step.
-template <typename ZT, bool MIXED>
-__global__ void __launch_bounds__(kBlock, 2) k_layer(NetDesc net, State st, int l, int i_begin, int prologue,
+template <typename ZT, bool MIXED, int WORDS>
+__global__ void __launch_bounds__(kBlock, 1) k_layer(NetDesc net, State st, int l, int i_begin, int prologue,
                                                      int mw) {
-  extern __shared__ double dsm[];
-  __shared__ Smem sm;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  Smem& sm = *reinterpret_cast<Smem*>(dsm);
+  double* ws = reinterpret_cast<double*>(dsm + kSmemBytes);
   if (cta_stopped(st)) return;
   unsigned int passed = 0;
   const int H = net.w[l + 1];
   if (threadIdx.x == 0) sm.nrl_layer = -1;
   __syncthreads();
   if (prologue) {
-    phase_decide<ZT, MIXED>(net, st, l, sm, dsm, mw);
+    phase_decide<ZT, MIXED>(net, st, l, sm, ws, mw);
     if (!grid_barrier(st.g, passed)) return;  // uniform per CTA
-    if (cta_stopped(st)) return;
     phase_scan0(net, st, l, sm);
     if (!grid_barrier(st.g, passed)) return;
-    if (cta_stopped(st)) return;
   }
   for (int i = i_begin; i < H; ++i) {
-    if (phase_step<ZT, MIXED>(net, st, l, i, sm, dsm, mw)) return;
-    if (!grid_barrier(st.g, passed)) return;
-    if (cta_stopped(st)) return;
+    if (phase_step<ZT, MIXED, WORDS>(net, st, l, i, sm, ws, mw)) return;  // every CTA takes the same decision
+    if (i + 1 < H && !grid_barrier(st.g, passed)) return;
   }
 }
 
@@ -414,6 +407,13 @@ __global__ void __launch_bounds__(kBlock) k_polish(NetDesc net, State st, float 
   if (lane == 0 && npol) atomic_add_ll(&st.g->polished, npol);
 }
 
+// rows[j][v] = Z[v][j]
+template <typename ZT>
+__global__ void k_value_rows(const ZT* Z, long long nV, int H, ZT* rows) {
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < nV * H; k += (long long)gridDim.x * blockDim.x)
+    rows[(k % H) * nV + k / H] = Z[k];
+}
+
 }  // namespace pc
 
 using namespace pc;
@@ -504,7 +504,7 @@ static void realloc_state(pc_ctx* c, long long V, long long E, long long T, bool
       if (rows && width) PC_CUDA(cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows, cudaMemcpyDeviceToDevice, c->stream));
     };
     cp2(nb.X, 8 * V, ob.X, 8 * oV, 8 * nV, D);
-    for (int k = 0; k < nb.nz && k < ob.nz; ++k) cp2(nb.Z[k], zs * V, ob.Z[k], zs * oV, zs * nV, Hm);
+    for (int k = 0; k < nb.nz && k < ob.nz; ++k) cp2(nb.Z[k], zs * Hm * V, ob.Z[k], zs * Hm * oV, zs * Hm * nV, 1);
     cp2(nb.esc, 4 * V, ob.esc, 4 * oV, 4 * nV, 1);
     cp2(nb.exc, 4 * V, ob.exc, 4 * oV, 4 * nV, 1);
     cp2(nb.SIG, 8 * V, ob.SIG, 8 * oV, 8 * nV, S);
@@ -632,7 +632,7 @@ struct Kernels {
     const int H = c->net.w[l + 1];
     if (c->opt.exec == PC_EXEC_PERSISTENT) {
       PC_CUDA(cudaMemsetAsync(&static_cast<Global*>(c->g)->barrier, 0, sizeof(unsigned int), c->stream));
-      auto fn = k_layer<ZT, MIXED>;
+      auto fn = c->net.S > 16 ? k_layer<ZT, MIXED, 2> : k_layer<ZT, MIXED, 1>;
       NetDesc net = c->net;
       State s = st;
       int l_ = l, ib = i_begin, pro = prologue ? 1 : 0, mw = c->mw;
@@ -641,19 +641,20 @@ struct Kernels {
                                           c->res_smem, c->stream));
       c->launches += 1;
     } else {
-      // grids sized to the edge capacity (2048 edges per CTA of a scan
-      // iteration), so that the small extractions of concurrent requests
-      // share the GPU; every phase is written for any grid size
-      const int gs = int(std::max<long long>(8, std::min<long long>(c->grid_step, c->Ecap / 2048)));
+      // grids sized to the edge capacity (4096 edges per CTA, which takes 32
+      // splits at a time), so that the small extractions of concurrent
+      // requests share the GPU; every phase is written for any grid size
+      const int gs = int(std::max<long long>(8, std::min<long long>(c->grid_step, c->Ecap / 4096)));
       if (prologue) {
         k_decide<ZT, MIXED><<<gs, kBlock, c->res_smem, c->stream>>>(c->net, st, l, c->mw);
         PC_CUDA(cudaGetLastError());
-        k_scan0<<<gs, kBlock, 0, c->stream>>>(c->net, st, l);
+        k_scan0<<<gs, kBlock, kSmemBytes, c->stream>>>(c->net, st, l);
         PC_CUDA(cudaGetLastError());
         c->launches += 2;
       }
       for (int i = i_begin; i < H; ++i) {
-        k_step<ZT, MIXED><<<gs, kBlock, c->res_smem, c->stream>>>(c->net, st, l, i, c->mw);
+        if (c->net.S > 16) k_step<ZT, MIXED, 2><<<gs, kBlock, c->res_smem, c->stream>>>(c->net, st, l, i, c->mw);
+        else k_step<ZT, MIXED, 1><<<gs, kBlock, c->res_smem, c->stream>>>(c->net, st, l, i, c->mw);
         PC_CUDA(cudaGetLastError());
         c->launches += 1;
       }
@@ -661,7 +662,10 @@ struct Kernels {
   }
   static int occupancy(pc_ctx* c) {
     int nb = 0;
-    PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_layer<ZT, MIXED>, kBlock, c->res_smem));
+    if (c->net.S > 16)
+      PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_layer<ZT, MIXED, 2>, kBlock, c->res_smem));
+    else
+      PC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_layer<ZT, MIXED, 1>, kBlock, c->res_smem));
     return nb;
   }
 };
@@ -914,11 +918,11 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
 
   // launch geometry
   net.rd_batch = rd_batch_size(mw, D, net.S);
-  c->res_smem = rd_layout(net.rd_batch, mw, D, net.S).total;
+  c->res_smem = kSmemBytes + (net.precision == PC_PREC_MIXED ? rd_layout(net.rd_batch, mw, D, net.S).total : 0);
   const int occ = occupancy_any(c);
   if (occ < 1) throw PcError(PC_ERR_INVALID, "persistent kernel does not fit on an SM");
   c->grid_persist = std::min(kMaxGrid, occ * c->num_sms);
-  c->grid_step = std::min(kMaxGrid, 2 * c->num_sms);
+  c->grid_step = std::min(kMaxGrid, c->num_sms);
 
   for (int k = 0; k <= pc_ctx::kPolishSlot; ++k) c->ev_used[k] = 0;
   if (dom) k_init_domain<<<1, 256, 0, c->stream>>>(net, make_state(c), X0dev, E0dev, dom->nv0, dom->ne0);
@@ -970,7 +974,7 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
     c->grows += 1;
   }
   if (c->deferred) {
-    k_verify_pairs<<<c->grid_step, 256, 0, c->stream>>>(net, make_state(c));
+    k_verify_pairs<<<8 * c->num_sms, 256, 0, c->stream>>>(net, make_state(c));
     PC_CUDA(cudaGetLastError());
     c->launches += 1;
   }
@@ -1089,15 +1093,22 @@ static cudaError_t set_func_attributes_now() {
     const cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) e = r;
   };
-  set((const void*)k_layer<double, false>, kRdSmemMax);
-  set((const void*)k_layer<float, false>, kRdSmemMax);
-  set((const void*)k_layer<float, true>, kRdSmemMax);
-  set((const void*)k_decide<double, false>, kRdSmemMax);
-  set((const void*)k_decide<float, false>, kRdSmemMax);
-  set((const void*)k_decide<float, true>, kRdSmemMax);
-  set((const void*)k_step<double, false>, kRdSmemMax);
-  set((const void*)k_step<float, false>, kRdSmemMax);
-  set((const void*)k_step<float, true>, kRdSmemMax);
+  set((const void*)k_layer<double, false, 1>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_layer<double, false, 2>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_layer<float, false, 1>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_layer<float, false, 2>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_layer<float, true, 1>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_layer<float, true, 2>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_decide<double, false>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_decide<float, false>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_decide<float, true>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_step<double, false, 1>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_step<double, false, 2>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_step<float, false, 1>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_step<float, false, 2>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_step<float, true, 1>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_step<float, true, 2>, kSmemBytes + kRdSmemMax);
+  set((const void*)k_scan0, kSmemBytes);
   set((const void*)k_polish<false>, kPolishSmemMax);
   set((const void*)k_polish<true>, kPolishSmemMax);
   {
@@ -1320,8 +1331,22 @@ pc_status pc_signvectors(pc_ctx* c, const uint64_t** dev, int64_t* ld, uint64_t*
 pc_status pc_values(pc_ctx* c, void* out) {
   if (!c) return PC_ERR_INVALID;
   if (!c->have_result) return c->fail(PC_ERR_INVALID, "no extraction result");
-  const int L = c->net.L;
-  return copy_rows(c, out, pc_make_state(c).Z[L - 1], zsize_of(c->net.precision), c->Vcap, c->nV, c->net.w[L]);
+  const int L = c->net.L, H = c->net.w[L];
+  const size_t zs = zsize_of(c->net.precision);
+  const void* Z = pc_make_state(c).Z[L - 1];
+  if (H == 1 || !out || c->nV == 0) return copy_rows(c, out, Z, zs, c->nV, c->nV, 1);
+  void* rows = ctx_alloc(c, zs * H * c->nV);  // the device keeps them vertex by vertex
+  if (!rows) return c->fail(PC_ERR_OOM, "values: device allocation failed");
+  const int grid = int(std::min<long long>(4096, (c->nV * H + 255) / 256));
+  if (zs == 8)
+    k_value_rows<double><<<grid, 256, 0, c->stream>>>(static_cast<const double*>(Z), c->nV, H, static_cast<double*>(rows));
+  else
+    k_value_rows<float><<<grid, 256, 0, c->stream>>>(static_cast<const float*>(Z), c->nV, H, static_cast<float*>(rows));
+  const cudaError_t e = cudaGetLastError();
+  const pc_status r = e == cudaSuccess ? copy_rows(c, out, rows, zs, c->nV, c->nV, H)
+                                       : c->fail(PC_ERR_CUDA, cudaGetErrorString(e));
+  ctx_free(c, rows);
+  return r;
 }
 
 pc_status pc_error_estimates(pc_ctx* c, float* value_scale, float* coord_rms) {
@@ -1532,9 +1557,9 @@ extern "C" pc_status pc_extract_noalloc(int L, const int32_t* widths, const doub
     PC_CUDA(cudaMemsetAsync(base + kNaOffTable, 0xff, 32 * kNaMaxT, c.stream));
     PC_CUDA(cudaMemsetAsync(base + kNaOffCnt, 0, sizeof(Counters) * (nn + 1), c.stream));
     net.rd_batch = rd_batch_size(mw, D, net.S);
-    c.res_smem = rd_layout(net.rd_batch, mw, D, net.S).total;
+    c.res_smem = kSmemBytes + (precision == PC_PREC_MIXED ? rd_layout(net.rd_batch, mw, D, net.S).total : 0);
     occupancy_any(&c);
-    c.grid_step = std::min(kMaxGrid, 2 * c.num_sms);
+    c.grid_step = std::min(kMaxGrid, c.num_sms);
     k_init<<<1, 256, 0, c.stream>>>(net, make_state(&c));
     PC_CUDA(cudaGetLastError());
     enqueue_any(&c, 0, 0, false);

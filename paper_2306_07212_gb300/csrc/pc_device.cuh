@@ -2,10 +2,11 @@
 //
 // State layout in HBM (structure of arrays, leading dimension = capacity):
 //   X     [D][Vcap]   float64 vertex coordinates
-//   Z     [H][Vcap]   current-layer pre-activations (float32, or float64 in
-//                     FP64 mode), neuron-major so one neuron's pass reads a
-//                     contiguous row; two buffers ping-pong across layers, or
-//                     one per layer when the interpolation tape is kept
+//   Z     [Vcap][H]   current-layer pre-activations (float32, or float64 in
+//                     FP64 mode), vertex-major with the layer's own width: a
+//                     split reads and writes whole rows; two buffers ping-pong
+//                     across layers, or one per layer when the interpolation
+//                     tape is kept
 //   esc   [Vcap]      float32 error scale rho of the vertex's FP32 Z column:
 //                     the rms error of z_j is about ||W_j||_2 rho + u/2 |b_j|
 //                     (FP32 and mixed precision)
@@ -48,7 +49,6 @@ constexpr unsigned long long kPaired64 = 1ull << 63;  // same, in the 16-byte sl
 constexpr int kBlock = 512;              // threads per CTA in the neuron phases
 constexpr int kWarps = kBlock / 32;
 constexpr int kMaxGrid = 1024;           // upper bound on CTAs of a phase grid
-constexpr int kFilterCap = 2 * kBlock;   // CTA-local list of filtered vertices
 
 // error bits in Global::error
 constexpr int kErrPairing = 1;
@@ -99,15 +99,15 @@ struct Counters {        // 128 bytes
   long long pad[6];
 };
 
-struct Global {
+struct alignas(8) Global {
+  unsigned int barrier;  // grid barrier arrival counter (reset per launch); 8-byte aligned, polled with error
+  int error;             // sticky kErr* bits
   int halted_at;         // -1, or the neuron whose step ran out of capacity
   int halt_reason;
-  int error;             // sticky kErr* bits
   int flips;             // FP64 re-decisions that changed the FP32 sign
   int flip_margin_bits;  // largest |z| / (FP32 error estimate) among them (float bits)
   int missed;            // audit band: wrong FP32 signs beyond kappa (not written back)
   int missed_margin_bits;
-  unsigned int barrier;  // grid barrier arrival counter (reset per launch)
   unsigned int barrier_extra;  // arrivals a barrier waits for beyond the grid: 0, or 1 to test the timeout path
   long long need_v, need_e, need_t;
   long long polished;
@@ -198,9 +198,9 @@ __device__ __forceinline__ long long atomic_add_ll(long long* p, long long x) {
   return (long long)atomicAdd(reinterpret_cast<unsigned long long*>(p), (unsigned long long)x);
 }
 
-__device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
-  unsigned int v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+__device__ __forceinline__ unsigned long long ld_acquire_u64(const void* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
 
@@ -216,32 +216,33 @@ __device__ __forceinline__ bool cta_stopped(const State& st) {
   return __syncthreads_or(threadIdx.x == 0 && stopped(st)) != 0;
 }
 
-// Grid-wide barrier for cooperative launches.  Bounded: after ~0.5 s of
-// waiting it sets kErrTimeout and returns false (the caller then exits).
-// With g->barrier_extra = 1 (a test of this path) the target is one arrival
-// beyond the grid, which never comes, and the limit is 4096 polls.
+// Grid-wide barrier for cooperative launches.  Bounded: after ~0.7 s of
+// polls it sets kErrTimeout and returns false (the caller then exits).  The
+// poll reads the error bits with the arrival counter (one 8-byte load), so a
+// fatal error of any CTA's earlier phases also returns false without another
+// round trip.  With g->barrier_extra = 1 (a test of the timeout) the target is
+// one arrival beyond the grid, which never comes, and the limit is 4096 polls.
 __device__ __forceinline__ bool grid_barrier(Global* g, unsigned int& passed) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     passed += 1;
-    const unsigned int extra = *(volatile unsigned int*)&g->barrier_extra;
-    const unsigned int target = passed * gridDim.x + extra;
-    const long long limit = extra ? (1ll << 12) : (1ll << 22);
     __threadfence();
     atomicAdd(&g->barrier, 1u);
-    int ok = 1;
-    long long spins = 0;
-    while (ld_acquire_u32(&g->barrier) < target) {
+    const unsigned int extra = *(volatile unsigned int*)&g->barrier_extra;
+    const unsigned int target = passed * gridDim.x + extra;
+    const int limit = extra ? (1 << 12) : (1 << 20);
+    unsigned long long x;
+    int spins = 0;
+    while (static_cast<unsigned int>(x = ld_acquire_u64(&g->barrier)) < target) {
       if (++spins > limit) {
         atomicOr(&g->error, kErrTimeout);
-        ok = 0;
+        x = static_cast<unsigned long long>(kErrTimeout) << 32;
         break;
       }
-      __nanosleep(64);
     }
     __threadfence();
-    s_ok = ok;
+    s_ok = (static_cast<int>(x >> 32) & kErrFatal) == 0;
   }
   __syncthreads();
   return s_ok != 0;

@@ -133,6 +133,46 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
   for (int q = 0; q < 16; ++q) r[q] = __uint_as_float(u[q]);
 }
 
+// The vertex's 32 inputs of chunk q: its row's values where positive (a value
+// is positive iff its sign entry is +), else 0.  16-byte loads when the rows
+// are 16-byte aligned.
+__device__ __forceinline__ void gather_chunk(const float* Zin, long long v, bool valid, int q, int K,
+                                             float (&x)[kTcChunkK]) {
+  const float* row = Zin + v * K + q * kTcChunkK;
+  const int left = valid ? K - q * kTcChunkK : 0;
+  if ((K & 3) == 0) {
+#pragma unroll
+    for (int g = 0; g < kTcChunkK / 4; ++g) {
+      const float4 z = 4 * g < left ? *reinterpret_cast<const float4*>(row + 4 * g) : make_float4(0.f, 0.f, 0.f, 0.f);
+      x[4 * g] = z.x;
+      x[4 * g + 1] = z.y;
+      x[4 * g + 2] = z.z;
+      x[4 * g + 3] = z.w;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < kTcChunkK; ++k) x[k] = k < left ? row[k] : 0.f;
+  }
+#pragma unroll
+  for (int k = 0; k < kTcChunkK; ++k) x[k] = x[k] > 0.f ? x[k] : 0.f;
+}
+
+// 16 outputs of a vertex's row, from neuron j0 (+ b_l).
+__device__ __forceinline__ void store_row16(float* row, int j0, int H, const float (&r)[16], const float* bias) {
+  if ((H & 3) == 0) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+      if (j0 + 4 * g < H)
+        *reinterpret_cast<float4*>(row + j0 + 4 * g) =
+            make_float4(r[4 * g] + bias[j0 + 4 * g], r[4 * g + 1] + bias[j0 + 4 * g + 1],
+                        r[4 * g + 2] + bias[j0 + 4 * g + 2], r[4 * g + 3] + bias[j0 + 4 * g + 3]);
+  } else {
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj)
+      if (j0 + jj < H) row[j0 + jj] = r[jj] + bias[j0 + jj];
+  }
+}
+
 // PIECES = 2: the 3xTF32 product (head x head + head x tail + tail x head);
 // each product keeps about 22 bits.  PIECES = 3: a three-piece split
 // (x = x0 + x1 + x2, which is exact for an FP32 x), with the six products
@@ -207,10 +247,8 @@ __global__ void __launch_bounds__(kTcTileM, 1) k_gemm_tc(NetDesc net, State st, 
   tc_fence_after();
   const uint32_t tmem = tmem_base;
   const uint32_t idesc = tf32_idesc(kTcTileM, Npad);
-  const long long Vcap = st.Vcap;
   const float* Zin = static_cast<const float*>(st.Z[l - 1]);
   float* Zout = static_cast<float*>(st.Z[l]);
-  const int ebase = net.m + net.off[l - 1];
   // buffer b's MMAs: committed (pending[b]) and the parity of their phase
   uint32_t parity[2] = {0u, 0u};
   int pending[2] = {0, 0};
@@ -223,23 +261,9 @@ __global__ void __launch_bounds__(kTcTileM, 1) k_gemm_tc(NetDesc net, State st, 
     for (int q = 0; q < KC && !fail; ++q) {
       // this vertex's 32 inputs of chunk q, masked by its activation pattern
       float x[kTcChunkK];
-      uint64_t word = 0;
-      int cw = -1;
+      gather_chunk(Zin, v, valid, q, K, x);
 #pragma unroll
-      for (int k0 = 0; k0 < kTcChunkK; ++k0) {
-        const int k = q * kTcChunkK + k0;
-        float a = 0.f;
-        if (valid && k < K) {
-          const int entry = ebase + k, wi = entry >> 5;
-          if (wi != cw) {
-            word = st.SIG[(long long)wi * Vcap + v];
-            cw = wi;
-          }
-          if (((word >> (2 * (entry & 31))) & 3ull) == kPlus) a = Zin[(long long)k * Vcap + v];
-        }
-        a2 = fmaf(a, a, a2);
-        x[k0] = a;
-      }
+      for (int k0 = 0; k0 < kTcChunkK; ++k0) a2 = fmaf(x[k0], x[k0], a2);
       for (int pa = PIECES - 1; pa >= 0; --pa) {  // tail pieces first
         const int b = stage;
         stage ^= 1;
@@ -310,11 +334,7 @@ __global__ void __launch_bounds__(kTcTileM, 1) k_gemm_tc(NetDesc net, State st, 
 #pragma unroll
         for (int jj = 0; jj < 16; ++jj) r[jj] += r2[jj];
       }
-      if (valid) {
-#pragma unroll
-        for (int jj = 0; jj < 16; ++jj)
-          if (j0 + jj < H) Zout[(long long)(j0 + jj) * Vcap + v] = r[jj] + bias[j0 + jj];
-      }
+      if (valid) store_row16(Zout + v * H, j0, H, r, bias);
     }
     if (valid) {
       // error scale of the layer's values: the rounding of the product
@@ -357,26 +377,6 @@ __global__ void __launch_bounds__(kTcTileM, 1) k_gemm_tc(NetDesc net, State st, 
 // where k_gemm_tc gives every K step its own accumulator.  Tensor memory
 // holds one chunk's accumulators (4 x 64 columns for layers up to 64 wide),
 // so two CTAs share an SM.
-__device__ __forceinline__ void gather_chunk(const State& st, const float* Zin, long long Vcap, long long v,
-                                             bool valid, int q, int K, int ebase, float (&x)[kTcChunkK]) {
-  uint64_t word = 0;
-  int cw = -1;
-#pragma unroll
-  for (int k0 = 0; k0 < kTcChunkK; ++k0) {
-    const int k = q * kTcChunkK + k0;
-    float a = 0.f;
-    if (valid && k < K) {
-      const int entry = ebase + k, wi = entry >> 5;
-      if (wi != cw) {
-        word = st.SIG[(long long)wi * Vcap + v];
-        cw = wi;
-      }
-      if (((word >> (2 * (entry & 31))) & 3ull) == kPlus) a = Zin[(long long)k * Vcap + v];
-    }
-    x[k0] = a;
-  }
-}
-
 template <int PIECES>
 __global__ void __launch_bounds__(kTcTileM, 2) k_gemm_tc2(NetDesc net, State st, int l, int Npad, int Kpad) {
   extern __shared__ unsigned char tc_raw[];
@@ -432,10 +432,8 @@ __global__ void __launch_bounds__(kTcTileM, 2) k_gemm_tc2(NetDesc net, State st,
   tc_fence_after();
   const uint32_t tmem = tmem_base;
   const uint32_t idesc = tf32_idesc(kTcTileM, Npad);
-  const long long Vcap = st.Vcap;
   const float* Zin = static_cast<const float*>(st.Z[l - 1]);
   float* Zout = static_cast<float*>(st.Z[l]);
-  const int ebase = net.m + net.off[l - 1];
   const int ng = Npad / 16;  // 16-column groups of the output
   uint32_t parity = 0u;
   float x[kTcChunkK];  // the chunk being split; the next one is gathered during the MMAs
@@ -447,7 +445,7 @@ __global__ void __launch_bounds__(kTcTileM, 2) k_gemm_tc2(NetDesc net, State st,
 #pragma unroll
     for (int j = 0; j < kTcMaxN; ++j) acc[j] = 0.f;
     float a2 = 0.f;
-    gather_chunk(st, Zin, Vcap, v, valid, 0, K, ebase, x);
+    gather_chunk(Zin, v, valid, 0, K, x);
     for (int q = 0; q < KC; ++q) {
       // the pieces of this chunk (the previous chunk's MMAs have completed)
 #pragma unroll
@@ -493,7 +491,7 @@ __global__ void __launch_bounds__(kTcTileM, 2) k_gemm_tc2(NetDesc net, State st,
         }
         mma_commit(&bar);
       }
-      if (q + 1 < KC) gather_chunk(st, Zin, Vcap, v, valid, q + 1, K, ebase, x);  // while the MMAs run
+      if (q + 1 < KC) gather_chunk(Zin, v, valid, q + 1, K, x);  // while the MMAs run
       if (!mbar_wait(&bar, parity)) fail = 1;
       parity ^= 1u;
       tc_fence_after();
@@ -517,9 +515,10 @@ __global__ void __launch_bounds__(kTcTileM, 2) k_gemm_tc2(NetDesc net, State st,
 #pragma unroll
       for (int g = 0; g < kTcMaxN / 16; ++g) {
         if (g >= ng) break;
+        float r[16];
 #pragma unroll
-        for (int jj = 0; jj < 16; ++jj)
-          if (g * 16 + jj < H) Zout[(long long)(g * 16 + jj) * Vcap + v] = acc[g * 16 + jj] + bias[g * 16 + jj];
+        for (int jj = 0; jj < 16; ++jj) r[jj] = acc[g * 16 + jj];
+        store_row16(Zout + v * H, g * 16, H, r, bias);
       }
       // error scale (as in k_gemm_tc with one accumulator per K step)
       const float u = 5.9604645e-8f;  // 2^-24

@@ -109,6 +109,93 @@ __device__ inline void newton_solve(const NetDesc& net, const State& st, long lo
   o.ok = 1;
 }
 
+// The system M x = r in float32 by one warp (lane r < D: row r of M and its
+// right-hand side; all lanes call it): Gauss-Jordan elimination with partial
+// pivoting.  Component d of the solution in lane d.  False when singular.
+__device__ inline bool solve_warp(int D, const float (&A)[kMaxD], float rhs, float& x) {
+  const int lane = threadIdx.x & 31;
+  float M[kMaxD];
+#pragma unroll
+  for (int c = 0; c < kMaxD; ++c) M[c] = A[c];
+  int var = -1;  // the column whose pivot this lane's row is
+  float diag = 1.f;
+#pragma unroll
+  for (int c = 0; c < kMaxD; ++c) {
+    if (c >= D) break;
+    const unsigned key = lane < D && var < 0 ? __float_as_uint(fabsf(M[c])) : 0u;
+    const unsigned top = __reduce_max_sync(0xffffffffu, key);
+    if (top == 0u) return false;  // uniform
+    const int piv = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
+    const float pv = __shfl_sync(0xffffffffu, M[c], piv);
+    if (lane == piv) {
+      var = c;
+      diag = pv;
+    }
+    const float f = lane == piv ? 0.f : M[c] / pv;
+#pragma unroll
+    for (int k = 0; k < kMaxD; ++k)
+      if (k > c && k < D) M[k] -= f * __shfl_sync(0xffffffffu, M[k], piv);
+    rhs -= f * __shfl_sync(0xffffffffu, rhs, piv);
+  }
+  const float mine = rhs / diag;
+  x = 0.f;
+  for (int c = 0; c < D; ++c) {
+    const int src = __ffs(__ballot_sync(0xffffffffu, var == c)) - 1;
+    const float y = __shfl_sync(0xffffffffu, mine, src);
+    if (lane == c) x = y;
+  }
+  return true;
+}
+
+// The same step with float64 accuracy by one warp (all lanes call it; the
+// zero set has D entries): a float32 solve and two float32 corrections of its
+// residual, which is formed in float64 (iterative refinement; each one gains
+// the accuracy of a float32 solve).  A float64 division takes ~2000 clocks
+// on this chip: an elimination in float64 took 9,500 clocks at D = 3.  dl: component of the step in lane d < D.  False
+// when the system is singular.
+__device__ inline bool newton_warp(const NetDesc& net, const State& st, long long v, const int* s_zl, const double* A,
+                                   const double* gv, double& dl) {
+  const int D = net.D, m = net.m, lane = threadIdx.x & 31;
+  double M[kMaxD];
+  float F[kMaxD];
+#pragma unroll
+  for (int c = 0; c < kMaxD; ++c) M[c] = 0.0;
+  double r = 0.0;
+  if (lane < D) {
+    const int j = s_zl[lane];
+    if (j < m) {
+      const int d = j >> 1;
+      const double xd = st.X[(long long)d * st.Vcap + v];
+#pragma unroll
+      for (int c = 0; c < kMaxD; ++c) M[c] = c == d ? ((j & 1) ? -1.0 : 1.0) : 0.0;
+      r = -((j & 1) ? (net.hi[d] - xd) : (xd - net.lo[d]));
+    } else {
+#pragma unroll
+      for (int c = 0; c < kMaxD; ++c)
+        if (c < D) M[c] = A[lane * D + c];
+      r = -gv[lane];
+    }
+  }
+  // rows scaled by an exact power of two, so that float32 holds them
+  int top = 0;
+#pragma unroll
+  for (int c = 0; c < kMaxD; ++c) top = max(top, __double2hiint(fabs(M[c])) >> 20);
+  const double scale = top > 0 && top < 2046 ? __hiloint2double((2046 - top) << 20, 0) : 1.0;
+#pragma unroll
+  for (int c = 0; c < kMaxD; ++c) F[c] = static_cast<float>(M[c] * scale);
+  dl = 0.0;
+  for (int it = 0; it < 3; ++it) {
+    float x;
+    if (!solve_warp(D, F, static_cast<float>(r * scale), x)) return false;
+    dl += static_cast<double>(x);
+    if (it == 2) break;
+#pragma unroll
+    for (int c = 0; c < kMaxD; ++c)
+      if (c < D) r = fma(-M[c], static_cast<double>(__shfl_sync(0xffffffffu, x, c)), r);
+  }
+  return true;
+}
+
 // ---------------------------------------------------------------------------
 // Float-float evaluation for the coordinate polish.
 //

@@ -262,6 +262,14 @@ __global__ void k_take_rows(T* base, long long ld, int rows, const int* order, l
     tmp[k] = base[(k / n) * ld + order[k % n]];
 }
 
+// The values' rows: tmp[i][j] = Z[order[i]][j], j < H.
+template <typename T>
+__global__ void k_take_items(const T* Z, const int* order, long long n, int H, T* tmp) {
+  const long long total = n * H;
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < total; k += (long long)gridDim.x * blockDim.x)
+    tmp[k] = Z[(long long)order[k / H] * H + k % H];
+}
+
 template <typename T>
 __global__ void k_put_rows(T* base, long long ld, int rows, const T* tmp, long long n) {
   const long long total = n * rows;
@@ -413,7 +421,15 @@ void pc_prune_vertices(pc_ctx* c) {
   };
   move(c->bufs.X, 8, c->net.D);
   move(c->bufs.SIG, 8, c->net.S);
-  move(st.Z[c->net.L - 1], zs, H);
+  void* Z = st.Z[c->net.L - 1];
+  if (kept > 0) {
+    const int g = grid_of((long long)kept * H);
+    if (zs == 8)
+      k_take_items<uint64_t><<<g, 256, 0, s>>>(static_cast<const uint64_t*>(Z), O, kept, H, static_cast<uint64_t*>(tmp));
+    else
+      k_take_items<uint32_t><<<g, 256, 0, s>>>(static_cast<const uint32_t*>(Z), O, kept, H, static_cast<uint32_t*>(tmp));
+    cudaMemcpyAsync(Z, tmp, zs * H * kept, cudaMemcpyDeviceToDevice, s);
+  }
   if (c->net.precision != PC_PREC_FP64) {
     move(c->bufs.esc, 4, 1);
     move(c->bufs.exc, 4, 1);
