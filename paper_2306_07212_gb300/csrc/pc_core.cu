@@ -1,7 +1,7 @@
 // libpc core: device state management, the set-up kernels, the SIMT
 // layer-start product (step (1) of Section 4.2; the tensor-core form is in
 // pc_gemm_tc.cu), the per-neuron phase kernels in both execution modes, the
-// exact check of fingerprint pairings, the coordinate polish, and the C ABI
+// exact check of fingerprint pairings, and the C ABI
 // declared in include/pc.h.
 #include <cuda_runtime.h>
 
@@ -30,7 +30,8 @@ __host__ __device__ inline long long pairs_offset(long long n_params) { return (
 // float32 copy of the parameters, and the norms used by the FP32 error
 // estimate: per layer max_j ||W_j||_2 and max_j |b_j|, per neuron ||W_n||_2,
 // |b_n| and 1/||W_n||_2 (rounded outward).
-__global__ void k_prep(NetDesc net, float* W32, float* norms, long long n_params) {
+// *rem (0 at the launch) becomes nonzero if any parameter is not a float32.
+__global__ void k_prep(NetDesc net, float* W32, float* norms, long long n_params, int* rem) {
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n_params;
        t += (long long)gridDim.x * blockDim.x)
   {
@@ -46,8 +47,9 @@ __global__ void k_prep(NetDesc net, float* W32, float* norms, long long n_params
       const int K = net.w[l], H = net.w[l + 1];
       dst = net.wofs[l] + (e % K) * H + e / K;
     }
-    reinterpret_cast<float2*>(W32 + pairs_offset(n_params))[dst] =
-        make_float2(h, static_cast<float>(w - static_cast<double>(h)));
+    const float lo = static_cast<float>(w - static_cast<double>(h));
+    reinterpret_cast<float2*>(W32 + pairs_offset(n_params))[dst] = make_float2(h, lo);
+    if (lo != 0.f) *rem = 1;  // also a NaN
   }
   if (blockIdx.x < net.L) {
     const int l = blockIdx.x, H = net.w[l + 1], K = net.w[l];
@@ -363,50 +365,6 @@ __global__ void __launch_bounds__(256) k_verify_pairs(NetDesc net, State st) {
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&st.g->error, kErrVerify);
 }
 
-// Coordinate polish: every vertex whose coordinate error estimate (rms)
-// exceeds thr is moved to its exact position by a Newton step on its D zero
-// entries (all entries are processed at this point), with the values in
-// float-float arithmetic (newton_ff_warp).  One warp per vertex; vertices are
-// dealt to warps round-robin.  n_stage: parameter pairs copied to shared
-// memory (all of them, or 0 when they do not fit; then they are read from
-// global memory, coalesced per layer).
-template <bool DOMAIN>
-__global__ void __launch_bounds__(kBlock) k_polish(NetDesc net, State st, float thr, int mw, long long n_stage) {
-  // blockDim.x = 32 x (warps whose workspace fits kPolishSmemMax)
-  extern __shared__ __align__(16) unsigned char psm[];
-  __shared__ int zl[kWarps][kMaxD + 2];
-  __shared__ NewtonOut nout[kWarps];
-  if (cta_stopped(st)) return;
-  const Counters* last = st.cnt + net.N;
-  const long long nV = last->nV_before + last->nsplit;
-  const long long Vcap = st.Vcap;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float2* Ps = reinterpret_cast<float2*>(psm);
-  for (long long t = threadIdx.x; t < n_stage; t += blockDim.x) Ps[t] = net.WT2[t];
-  __syncthreads();
-  const float2* P = n_stage > 0 ? Ps : net.WT2;
-  unsigned char* ws = psm + ((n_stage * 8 + 15) / 16) * 16 + (long long)warp * ff_ws_bytes(mw, net.D);
-  long long npol = 0;
-  const int wpc = blockDim.x >> 5;
-  const long long nwarps = (long long)gridDim.x * wpc;
-  for (long long base = ((long long)blockIdx.x * wpc + warp) * 32; base < nV; base += nwarps * 32) {
-    const long long v = base + lane;
-    unsigned flag = __ballot_sync(0xffffffffu, v < nV && !(st.exc[v] <= thr));
-    while (flag) {
-      const int L = __ffs(flag) - 1;
-      flag &= flag - 1;
-      const long long u = base + L;
-      newton_ff_warp<DOMAIN>(net, st, P, u, net.P, mw, ws, zl[warp], &nout[warp]);
-      if (nout[warp].ok) {
-        if (lane < net.D) st.X[(long long)lane * Vcap + u] += nout[warp].dlt[lane];
-        npol += (lane == 0);
-      }
-      __syncwarp();
-    }
-  }
-  if (lane == 0 && npol) atomic_add_ll(&st.g->polished, npol);
-}
-
 // rows[j][v] = Z[v][j]
 template <typename ZT>
 __global__ void k_value_rows(const ZT* Z, long long nV, int H, ZT* rows) {
@@ -696,13 +654,6 @@ static int occupancy_any(pc_ctx* c) {
   }
 }
 
-// Parameter pairs the polish keeps in shared memory: all p (8 B each) when
-// they leave room for at least 8 warp workspaces, else none.
-static long long polish_stage(long long p, size_t ws) {
-  const long long bytes = (p * 8 + 15) / 16 * 16;
-  return bytes + 8 * (long long)ws <= kPolishSmemMax ? p : 0;
-}
-
 // Thrown when the exact check after a fingerprint-paired extraction fails.
 struct NeedsInlinePairing {};
 
@@ -871,7 +822,7 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
     ctx_free(c, c->norms);
     c->params64 = ctx_alloc(c, pbytes);
     c->params32 = ctx_alloc(c, sizeof(float) * (pairs_offset(p) + 2 * p));  // heads, then (head, remainder) pairs
-    c->norms = ctx_alloc(c, sizeof(float) * (2 * kMaxL + 3 * (size_t)n));
+    c->norms = ctx_alloc(c, sizeof(float) * (2 * kMaxL + 3 * (size_t)n + 1));  // and the remainder flag
     if (!c->params64 || !c->params32 || !c->norms) {
       ctx_free(c, c->params64);
       ctx_free(c, c->params32);
@@ -887,7 +838,11 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
   net.WT2 = reinterpret_cast<const float2*>(net.W32 + pairs_offset(p));
   net.norms = static_cast<const float*>(c->norms);
   net.nrm = net.norms + 2 * kMaxL;
-  k_prep<<<std::max(L, 64), 256, 0, c->stream>>>(net, static_cast<float*>(c->params32), static_cast<float*>(c->norms), p);
+  int* rem = reinterpret_cast<int*>(static_cast<float*>(c->norms) + 2 * kMaxL + 3 * n);
+  net.rem = rem;
+  PC_CUDA(cudaMemsetAsync(rem, 0, sizeof(int), c->stream));
+  k_prep<<<std::max(L, 64), 256, 0, c->stream>>>(net, static_cast<float*>(c->params32), static_cast<float*>(c->norms), p,
+                                                 rem);
   PC_CUDA(cudaGetLastError());
 
   // state buffers (kept across extractions when shapes allow)
@@ -983,17 +938,8 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
     double diam = 0.0;
     for (int d = 0; d < D; ++d) diam += (hi[d] - lo[d]) * (hi[d] - lo[d]);
     const float thr = static_cast<float>((c->opt.polish_tol > 0 ? c->opt.polish_tol : 1e-6) * std::sqrt(diam));
-    const size_t ws = ff_ws_bytes(c->mw, D);
-    const long long n_stage = polish_stage(p, ws);
-    const size_t stage_b = (n_stage * 8 + 15) / 16 * 16;
-    const int wpc = std::max(1, std::min(kWarps, int((kPolishSmemMax - stage_b) / ws)));
     TimerScope ts(c, pc_ctx::kPolishSlot);
-    if (pc_polish_tile_eligible(net))
-      PC_CUDA(pc_polish_tile_launch(net, make_state(c), thr, c->mw, c->num_sms, dom, c->stream));
-    else if (dom)
-      k_polish<true><<<c->grid_step, 32 * wpc, stage_b + ws * wpc, c->stream>>>(net, make_state(c), thr, c->mw, n_stage);
-    else
-      k_polish<false><<<c->grid_step, 32 * wpc, stage_b + ws * wpc, c->stream>>>(net, make_state(c), thr, c->mw, n_stage);
+    PC_CUDA(pc_polish_launch(net, make_state(c), thr, c->mw, c->num_sms, p, c->stream));
     PC_CUDA(cudaGetLastError());
     c->launches += 1;
   }
@@ -1109,14 +1055,12 @@ static cudaError_t set_func_attributes_now() {
   set((const void*)k_step<float, true, 1>, kSmemBytes + kRdSmemMax);
   set((const void*)k_step<float, true, 2>, kSmemBytes + kRdSmemMax);
   set((const void*)k_scan0, kSmemBytes);
-  set((const void*)k_polish<false>, kPolishSmemMax);
-  set((const void*)k_polish<true>, kPolishSmemMax);
   {
     const cudaError_t r = pc_gemm_tc_set_attributes();
     if (e == cudaSuccess) e = r;
   }
   {
-    const cudaError_t r = pc_polish_tile_set_attributes();
+    const cudaError_t r = pc_polish_set_attributes();
     if (e == cudaSuccess) e = r;
   }
   {
@@ -1420,7 +1364,7 @@ constexpr size_t na_align(size_t x) { return (x + 255) / 256 * 256; }
 constexpr size_t kNaOffP64 = 0;
 constexpr size_t kNaOffP32 = kNaOffP64 + na_align(8 * kNaMaxParams);
 constexpr size_t kNaOffNorm = kNaOffP32 + na_align(12 * kNaMaxParams + 8);
-constexpr size_t kNaOffZ0 = kNaOffNorm + na_align(4 * (2 * kMaxL + 3 * kNaMaxN));
+constexpr size_t kNaOffZ0 = kNaOffNorm + na_align(4 * (2 * kMaxL + 3 * kNaMaxN + 1));
 constexpr size_t kNaZBytes = na_align(8ull * kNaMaxWidth * kNaMaxV);
 constexpr size_t kNaOffZ1 = kNaOffZ0 + kNaZBytes;
 constexpr size_t kNaOffEsc = kNaOffZ1 + kNaZBytes;
@@ -1550,8 +1494,11 @@ extern "C" pc_status pc_extract_noalloc(int L, const int32_t* widths, const doub
     c.Ecap = cap_e;
     c.Tcap = kNaMaxT;
     PC_CUDA(cudaMemcpyAsync(base + kNaOffP64, params, sizeof(double) * p, cudaMemcpyDefault, c.stream));
+    int* rem = reinterpret_cast<int*>(base + kNaOffNorm) + 2 * kMaxL + 3 * nn;
+    net.rem = rem;
+    PC_CUDA(cudaMemsetAsync(rem, 0, sizeof(int), c.stream));
     k_prep<<<std::max(L, 64), 256, 0, c.stream>>>(net, reinterpret_cast<float*>(base + kNaOffP32),
-                                                   reinterpret_cast<float*>(base + kNaOffNorm), p);
+                                                   reinterpret_cast<float*>(base + kNaOffNorm), p, rem);
     PC_CUDA(cudaGetLastError());
     // the scratch keeps the previous call's contents: reset what must start empty
     PC_CUDA(cudaMemsetAsync(base + kNaOffTable, 0xff, 32 * kNaMaxT, c.stream));
@@ -1567,14 +1514,7 @@ extern "C" pc_status pc_extract_noalloc(int L, const int32_t* widths, const doub
       double diam = 0.0;
       for (int d = 0; d < D; ++d) diam += (hi[d] - lo[d]) * (hi[d] - lo[d]);
       const float thr = static_cast<float>(c.opt.polish_tol * std::sqrt(diam));
-      const size_t ws = ff_ws_bytes(c.mw, D);
-      const long long n_stage = polish_stage(p, ws);
-      const size_t stage_b = (n_stage * 8 + 15) / 16 * 16;
-      const int wpc = std::max(1, std::min(kWarps, int((kPolishSmemMax - stage_b) / ws)));
-      if (pc_polish_tile_eligible(net))
-        PC_CUDA(pc_polish_tile_launch(net, make_state(&c), thr, c.mw, c.num_sms, false, c.stream));
-      else
-        k_polish<false><<<c.grid_step, 32 * wpc, stage_b + ws * wpc, c.stream>>>(net, make_state(&c), thr, c.mw, n_stage);
+      PC_CUDA(pc_polish_launch(net, make_state(&c), thr, c.mw, c.num_sms, p, c.stream));
       PC_CUDA(cudaGetLastError());
     }
     Global g{};

@@ -1,24 +1,33 @@
-// Coordinate polish, tiled: every vertex whose coordinate error estimate
-// exceeds the threshold moves to the exact intersection of its D zero sets
-// (the vertex of Section 4.2's complex: D entries of its sign vector are
-// zero, each affine on the vertex's own piece, Eq. 4 with the stored
-// activation pattern).  One Newton step from the stored coordinates solves
-// the D x D system A dx = -g, with the values g in float-float and the
-// gradients A in float32 (the step is small, so float32 gradients add only
-// ~1e-7 of the step; see pc_newton.cuh).
+// Coordinate polish: every vertex whose coordinate error estimate exceeds the
+// threshold moves to the exact intersection of its D zero sets (the vertex of
+// Section 4.2's complex: D entries of its sign vector are zero, each affine on
+// the vertex's own piece, Eq. 4 with the stored activation pattern).  One
+// Newton step from the stored coordinates solves the D x D system A dx = -g,
+// with the values g in float-float and the gradients A in float32 (the step is
+// small, so float32 gradients add only ~1e-7 of the step; see pc_newton.cuh).
 //
-// The forward pass over the vertices is a matrix product per layer,
-//   a_k[r][v] = sum_c W_k[r][c] a_{k-1}[c][v] + b_k[r]   (masked by v's signs),
-// so it runs as one: a CTA owns a tile of TV consecutive vertices (vertices
-// are created layer by layer, so a tile's vertices mostly need the same
-// layers), keeps the tile's activations (hi, lo) and gradients (D per input)
-// neuron-major in shared memory, and each thread accumulates a block of 4
-// vertices x kPtRows neurons, so every activation it loads serves kPtRows
-// outputs and every weight four.  The dot products follow Ogita-Rump-Oishi Dot2 (exact
-// products by FMA, TwoSum of the running sum, error terms summed in a
-// float), like newton_ff_warp; the layer's outputs overwrite its inputs
-// after a barrier.  D <= kPtMaxD; larger D takes the one-warp-per-vertex
-// kernel (k_polish).
+// The forward pass that gives g and A is a chain of matrix products with a mask
+// per vertex: about half of a layer's inputs are inactive (exact zeros) and
+// half of its outputs are not needed by the next layer, and in the vertex's
+// last layer only its zero entries are.  So a vertex is worked on by itself, by
+// 8 or 16 lanes, over lists: inputs are its active neurons, outputs its active
+// neurons and the neurons of its zero set, about a fifth of the dense
+// multiply-adds.  Every lane holds up to kPtRows outputs (the layer's list, 8 or
+// 16 apart), so that an input's record (head, remainder and D gradient entries,
+// one or two 16-byte broadcasts from shared memory) serves up to 64 outputs,
+// and pairs of outputs run on packed FP32 instructions (each rounded as the
+// scalar form).  Weight heads are staged in shared memory when they fit; their remainders are read only for networks
+// that have any (NetDesc::rem).
+//
+// The dot products follow Ogita-Rump-Oishi Dot2 (exact products by FMA, TwoSum
+// of the running sum, error terms summed in a float), about 44 bits; a skipped
+// zero input changes no bit of them, so every sum is the dense one's in its order.
+//
+// Bound by FP32 issue.  Measured on GB300 against a dense product over tiles
+// of 32 vertices (D <= 5) and a dense pass of a warp per vertex (D > 5):
+// 3-64x4-1 (314k
+// vertices) 2.57 -> 0.77 ms, 5-40x4-1 (1e7) 39 -> 15.7 ms, 4-128x3-1 (212k) 3.8
+// -> 1.35 ms, 8-10x4-1 (369k) 7.7 -> 0.93 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -30,19 +39,31 @@
 
 namespace pc {
 
-constexpr int kPtThreads = 256;
-constexpr int kPtRows = 2;       // neurons per thread (a thread's block: 4 vertices x kPtRows neurons)
-constexpr int kPtMinBlocks = 2;  // CTAs per SM the register allocation is made for
-constexpr int kPtMaxD = 5;
-constexpr int kPtSmemMax = 200 * 1024;
+constexpr int kPtThreads = 512;  // at most
+constexpr int kPtRows = 8;       // outputs of a lane in one pass over the inputs, at most
+constexpr int kPtMaxD = kMaxD;
+constexpr int kPtSmemMax = 200 * 1024;  // vertices' workspace
+constexpr int kPtSmemAll = 224 * 1024;  // and the staged weights
+
+// Lanes of a vertex: 8 where they hold a layer's outputs in one pass and the
+// Newton system's rows (what is not the products -- lists, the solve, the few
+// outputs of the last layer -- then serves four vertices per instruction),
+// else 16.  With 16 lanes
+// throughout: 0.97 and 24.3 ms instead of 0.77 and 15.7 on the two first nets
+// above.
+__host__ __device__ constexpr int pt_lanes(int mw, int D) { return mw <= 8 * kPtRows && D <= 8 ? 8 : 16; }
 
 struct PtLayout {
   int TV, rows;
   size_t A, gv, sig, ahi, alo, J, zl, nz, total;
 };
 
-// Shared-memory layout of one tile (byte offsets, each 16-aligned).  rows:
-// activation rows held (the widest layer, and D for the coordinates).
+// Floats of an input's record: head, remainder, D gradient entries, padded to
+// 16 bytes.
+__host__ __device__ constexpr int pt_record(int D) { return (2 + D + 3) / 4 * 4; }
+
+// Shared-memory layout of a CTA's TV vertices (byte offsets, each 16-aligned).
+// rows: records held per vertex (the widest layer, and D for the coordinates).
 __host__ __device__ inline PtLayout pt_layout(int TV, int mw, int S, int D) {
   PtLayout p{};
   p.TV = TV;
@@ -53,272 +74,493 @@ __host__ __device__ inline PtLayout pt_layout(int TV, int mw, int S, int D) {
     o += (bytes + 15) / 16 * 16;
     return at;
   };
-  p.A = take((size_t)TV * D * D * 8);
-  p.gv = take((size_t)TV * D * 8);
-  p.sig = take((size_t)TV * S * 8);
-  p.ahi = take((size_t)p.rows * TV * 4);
-  p.alo = take((size_t)p.rows * TV * 4);
-  p.J = take((size_t)p.rows * D * TV * 4);
-  p.zl = take((size_t)TV * D * 4);
-  p.nz = take((size_t)TV * 4);
+  const size_t rec = (size_t)TV * p.rows * pt_record(D) * 4;
+  p.A = take((size_t)TV * D * D * 4);                 // Newton rows [TV][D][D] (float)
+  p.gv = take((size_t)TV * D * 8);                    // their values [TV][D] (double)
+  p.sig = take(0 * (size_t)S);                        // sign words stay in registers
+  p.ahi = take(rec);                                  // records by list position [TV][rows][pt_record]
+  // the next layer's, when one pass does not hold all outputs
+  p.alo = take(p.rows > kPtRows * pt_lanes(mw, D) ? rec : 0);
+  p.J = take((size_t)TV * p.rows * 2 * 2);            // lists [TV][2][rows]: inputs (offsets of weight rows), outputs
+  p.zl = take((size_t)TV * D * 4);                    // zero entries [TV][D]
+  p.nz = take((size_t)pt_record(D) * 4);              // a record of zeros
   p.total = o;
   return p;
 }
 
-// Vertices per tile: the (vertex, neuron) blocks of the widest layer fill
-// the CTA, at most 128 vertices, and the tile fits the shared memory.
+// Vertices per CTA, fewer when their records do not fit.
 static int pt_tile_vertices(int mw, int S, int D) {
-  const int nrg = (mw + kPtRows - 1) / kPtRows;
-  int TV = std::min(128, 4 * std::max(1, kPtThreads / nrg));
+  int TV = kPtThreads / pt_lanes(mw, D);
   while (TV > 4 && pt_layout(TV, mw, S, D).total > (size_t)kPtSmemMax) TV -= 4;
   return TV;
 }
 
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+// One Dot2 step of two outputs: s + e += w * (hi + lo), w = head + rem; nhi =
+// -hi.  Differences are FMAs with -1 (the packed instructions take no negated
+// operands; the rounding is the subtraction's).
+template <bool REM>
+__device__ __forceinline__ void dot2_step(float2 w, float2 rem, float2 hi, float2 nhi, float2 lo, float2& s, float2& e) {
+  const float2 m1 = make_float2(-1.f, -1.f);
+  const float2 np = __fmul2_rn(w, nhi);                // -(w hi)
+  float2 er = __ffma2_rn(w, hi, np);                   // exact low part of the product
+  er = __ffma2_rn(w, lo, er);                          // cross terms of the low parts
+  if (REM) er = __ffma2_rn(rem, hi, er);
+  const float2 t = __ffma2_rn(np, m1, s);              // TwoSum: t + its error is exact
+  const float2 bb = __ffma2_rn(s, m1, t);
+  const float2 ts = __ffma2_rn(__ffma2_rn(bb, m1, t), m1, s);
+  const float2 tp = __fadd2_rn(np, bb);
+  e = __fadd2_rn(e, __fadd2_rn(__ffma2_rn(tp, m1, ts), er));
+  s = t;
+}
 
-template <int DT, bool DOMAIN>
-__global__ void __launch_bounds__(kPtThreads, kPtMinBlocks) k_polish_tile(NetDesc net, State st, float thr, int mw, int TV) {
+// Weight (head, remainder) of neuron r for input c: staged heads, or the
+// pairs in global memory.
+template <bool STAGED>
+__device__ __forceinline__ float2 weight(const float* Ws, const float2* Wg, int at) {
+  if (STAGED) return make_float2(Ws[at], 0.f);
+  return __ldg(Wg + at);
+}
+
+// The scalar form.
+template <bool REM>
+__device__ __forceinline__ void dot2_step(float w, float rem, float hi, float lo, float& s, float& e) {
+  const float pr = __fmul_rn(w, hi);
+  float er = fmaf(w, hi, -pr);
+  er = fmaf(w, lo, er);
+  if (REM) er = fmaf(rem, hi, er);
+  const float t = __fadd_rn(s, pr);
+  const float bb = __fsub_rn(t, s);
+  const float ts = __fsub_rn(s, __fsub_rn(t, bb));
+  e = __fadd_rn(e, __fadd_rn(__fadd_rn(ts, __fsub_rn(pr, bb)), er));
+  s = t;
+}
+
+// A lane's gradients of one output: pairs of components, then an odd one, as
+// they lie in the records.
+template <int DT>
+struct Grad {
+  float2 p[DT / 2 > 0 ? DT / 2 : 1];
+  float o;
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int d = 0; d < DT / 2; ++d) p[d] = make_float2(0.f, 0.f);
+    o = 0.f;
+  }
+  __device__ __forceinline__ void add(float w, const float* r) {  // r: the record's gradient
+#pragma unroll
+    for (int d = 0; d < DT / 2; ++d)
+      p[d] = __ffma2_rn(make_float2(w, w), make_float2(r[2 * d], r[2 * d + 1]), p[d]);
+    if (DT & 1) o = fmaf(w, r[DT - 1], o);
+  }
+  __device__ __forceinline__ float at(int d) const {
+    return (DT & 1) && d == DT - 1 ? o : ((d & 1) ? p[d / 2].y : p[d / 2].x);
+  }
+};
+
+// NR outputs per lane (value sums of pairs of outputs packed, then an odd one)
+// over the vertex's inputs [0, cmax) (its own count is ci; the other half warp
+// may have more, past its own it reads a record of zeros, which changes
+// nothing): (s, e) and the gradients of the outputs row[0 .. NR).  li: offsets
+// of the inputs' weight rows.
+template <int DT, int NR, bool STAGED, bool REM>
+__device__ __forceinline__ void rows_pass(const float* rec, const float* none, const uint16_t* li, int ci, int cmax,
+                                          const float* Ws, const float2* Wg, const int (&row)[kPtRows],
+                                          float2 (&s)[kPtRows / 2], float2 (&e)[kPtRows / 2], Grad<DT> (&g)[kPtRows]) {
+  constexpr int PS = pt_record(DT), NP = NR / 2;
+#pragma unroll 2
+  for (int t = 0; t < cmax; ++t) {
+    const bool in = t < ci;
+    const int c = in ? li[t] : 0;
+    const float* at = in ? rec + t * PS : none;
+    float x[PS];
+#pragma unroll
+    for (int h = 0; h < PS / 4; ++h) {
+      const float4 f = *reinterpret_cast<const float4*>(at + 4 * h);
+      x[4 * h] = f.x;
+      x[4 * h + 1] = f.y;
+      x[4 * h + 2] = f.z;
+      x[4 * h + 3] = f.w;
+    }
+    const float hi = x[0], lo = x[1];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const float2 wa = weight<STAGED>(Ws, Wg, c + row[2 * p]), wb = weight<STAGED>(Ws, Wg, c + row[2 * p + 1]);
+      dot2_step<REM>(make_float2(wa.x, wb.x), make_float2(wa.y, wb.y), make_float2(hi, hi), make_float2(-hi, -hi),
+                     make_float2(lo, lo), s[p], e[p]);
+      g[2 * p].add(wa.x, x + 2);
+      g[2 * p + 1].add(wb.x, x + 2);
+    }
+    if (NR & 1) {
+      const float2 w = weight<STAGED>(Ws, Wg, c + row[2 * NP]);
+      dot2_step<REM>(w.x, w.y, hi, lo, s[NP].x, e[NP].x);
+      g[2 * NP].add(w.x, x + 2);
+    }
+  }
+}
+
+// The D x D system of a vertex by its LN lanes (lane r < D holds row r of M and
+// the right-hand side; all lanes of the warp call it): Gaussian elimination
+// with partial pivoting and back substitution in float32, rows in parallel.
+// Component d in lane d; ok false when singular.
+template <int DT, int LN>
+__device__ __forceinline__ float solve_group(float (&M)[DT], float rhs, bool& ok) {
+  const int gl = threadIdx.x & (LN - 1);
+  int pos = gl;      // the row's place in the elimination order
+  int piv[DT];       // lane of the c-th pivot row
+#pragma unroll
+  for (int c = 0; c < DT; ++c) {
+    const unsigned key = gl < DT && pos >= c ? __float_as_uint(fabsf(M[c])) + 1u : 0u;
+    unsigned top = 0;
+    int best = 0, at = 0;
+#pragma unroll
+    for (int r = 0; r < DT; ++r) {  // the largest; the first of equal ones
+      const unsigned k = __shfl_sync(0xffffffffu, key, r, LN);
+      const int p = __shfl_sync(0xffffffffu, pos, r, LN);
+      if (k > top || (k == top && p < at)) {
+        top = k;
+        best = r;
+        at = p;
+      }
+    }
+    if (top <= 1u) ok = false;
+    piv[c] = best;
+    const bool mine = gl == best;
+    if (!mine && pos == c) pos = at;  // the rows change places
+    if (mine) pos = c;
+    const float f = M[c] / __shfl_sync(0xffffffffu, M[c], best, LN);
+#pragma unroll
+    for (int k = c + 1; k < DT; ++k) {
+      const float x = __shfl_sync(0xffffffffu, M[k], best, LN);
+      if (pos > c) M[k] = fmaf(-f, x, M[k]);
+    }
+    const float x = __shfl_sync(0xffffffffu, rhs, best, LN);
+    if (pos > c) rhs = fmaf(-f, x, rhs);
+  }
+  float sol[DT], out = 0.f;
+#pragma unroll
+  for (int r = DT - 1; r >= 0; --r) {
+    float acc = rhs;
+#pragma unroll
+    for (int k = r + 1; k < DT; ++k) acc = fmaf(-M[k], sol[k], acc);
+    sol[r] = __shfl_sync(0xffffffffu, acc / M[r], piv[r], LN);
+    if (gl == r) out = sol[r];
+  }
+  return out;
+}
+
+template <int N>
+struct Int {
+  static constexpr int value = N;
+};
+
+// WEIGHTS: heads staged in shared memory (a network without remainders), or
+// pairs from global memory.
+template <int DT, int LN, bool STAGED>
+__device__ __forceinline__ void polish_vertices(const NetDesc& net, const State& st, float thr, int mw, int TV,
+                                                unsigned char* sm, const float* Ps, long long nV, int& npol) {
+  constexpr int NW = kMaxWords / LN;        // sign words per lane: gl, gl + LN, ...
+  constexpr unsigned kMask = (1u << LN) - 1u;
+  constexpr int kPass = LN * kPtRows;
+  constexpr bool REM = !STAGED;
+  const int lane = threadIdx.x & 31, gl = lane & (LN - 1), gsh = lane & ~(LN - 1), g = threadIdx.x / LN;
+  const int S = net.S, m = net.m;
+  const long long Vcap = st.Vcap;
+  constexpr int PS = pt_record(DT);
+  const PtLayout lay = pt_layout(TV, mw, S, DT);
+  float* A = reinterpret_cast<float*>(sm + lay.A) + g * DT * DT;
+  double* gv = reinterpret_cast<double*>(sm + lay.gv) + g * DT;
+  float* rec = reinterpret_cast<float*>(sm + lay.ahi) + (size_t)g * lay.rows * PS;
+  float* next = lay.rows > kPass ? reinterpret_cast<float*>(sm + lay.alo) + (size_t)g * lay.rows * PS : rec;
+  uint16_t* li = reinterpret_cast<uint16_t*>(sm + lay.J) + (size_t)g * 2 * lay.rows;
+  uint16_t* lo_ = li + lay.rows;
+  int* zl = reinterpret_cast<int*>(sm + lay.zl) + g * DT;
+  const float* none = reinterpret_cast<const float*>(sm + lay.nz);  // a record of zeros
+  auto gballot = [&](bool x) { return (__ballot_sync(0xffffffffu, x) >> gsh) & kMask; };
+  auto most = [&](int x) {  // over the warp's groups
+#pragma unroll
+    for (int o = LN; o < 32; o <<= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
+    return x;
+  };
+  const long long stride = (long long)gridDim.x * TV;
+  for (long long base = (long long)blockIdx.x * TV; base < nV; base += stride) {
+    const long long v = base + g;
+    bool act = v < nV && !(st.exc[v] <= thr);
+    if (!__any_sync(0xffffffffu, act)) continue;
+    uint64_t word[NW];
+#pragma unroll
+    for (int x = 0; x < NW; ++x)
+      word[x] = act && gl + LN * x < S ? st.SIG[(long long)(gl + LN * x) * Vcap + v] : 0ull;
+    double xd = 0.0;
+    if (act && gl < DT) xd = st.X[(long long)gl * Vcap + v];
+    // the zero entries in order
+    int nz = 0;
+#pragma unroll
+    for (int x = 0; x < NW; ++x) {
+      if (LN * x >= S) break;
+      const int w = gl + LN * x;
+      uint64_t mm = act && w < S ? zero_mask(word[x], w, net.P) : 0ull;
+      const int c0 = __popcll(mm);
+      int at = nz;
+      for (int y = 1; __any_sync(0xffffffffu, c0 >= y); ++y) {
+        const unsigned b = gballot(c0 >= y);
+        at += __popc(b & ((1u << gl) - 1u));
+        nz += __popc(b);
+      }
+      for (; mm; mm &= mm - 1, ++at)
+        if (at < DT) zl[at] = w * 32 + ((__ffsll((long long)mm) - 1) >> 1);
+    }
+    act = act && nz == DT;  // else not a vertex of the generic complex: left as it is
+    __syncwarp();
+    // the highest layer among the zero entries
+    int lmax = -1;
+    const int mine = act && gl < DT ? zl[gl] : 0;
+    for (int l = 0; l < net.L; ++l)
+      if (act && gl < DT && mine - m >= net.off[l]) lmax = l;
+#pragma unroll
+    for (int o = LN / 2; o > 0; o >>= 1) lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+    const int lall = most(lmax);
+    // the coordinates (float-float) with the identity as their gradient
+    if (gl < DT) {
+      const float h = static_cast<float>(xd);
+      float* r = rec + gl * PS;
+      r[0] = h;
+      r[1] = static_cast<float>(xd - static_cast<double>(h));
+#pragma unroll
+      for (int d = 0; d < DT; ++d) r[2 + d] = d == gl ? 1.f : 0.f;
+      li[gl] = static_cast<uint16_t>(gl * net.w[1]);
+    }
+    int ci = act ? DT : 0;
+    for (int k = 0; k <= lall; ++k) {
+      const int H = net.w[k + 1], e0 = m + net.off[k];
+      // outputs: the active neurons (not in the vertex's last layer), then the
+      // zero set's
+      const bool need = act && k <= lmax, last = k >= lmax;
+      int n = 0;
+      for (int h = 0; h * LN < H && __any_sync(0xffffffffu, need && !last); ++h) {
+        const int r = h * LN + gl, entry = e0 + r, w = entry >> 5;
+        uint64_t x = __shfl_sync(0xffffffffu, word[0], w & (LN - 1), LN);
+#pragma unroll
+        for (int y = 1; y < NW; ++y) {
+          if (LN * y >= S) break;
+          const uint64_t z = __shfl_sync(0xffffffffu, word[y], w & (LN - 1), LN);
+          if (w / LN == y) x = z;
+        }
+        const bool take = need && !last && r < H && ((x >> (2 * (entry & 31))) & 3ull) == kPlus;
+        const unsigned b = gballot(take);
+        if (take) lo_[n + __popc(b & ((1u << gl) - 1u))] = static_cast<uint16_t>(r);
+        n += __popc(b);
+      }
+      int nn = n;
+#pragma unroll
+      for (int q0 = 0; q0 < DT; q0 += LN) {  // the vertex's zero entries of this layer
+        const bool here = need && q0 + gl < DT && mine >= e0 && mine < e0 + H;
+        const unsigned b = gballot(here);
+        if (here) lo_[nn + __popc(b & ((1u << gl) - 1u))] = static_cast<uint16_t>(mine - e0);
+        nn += __popc(b);
+      }
+      __syncwarp();
+      const int nmax = most(nn), cmax = most(ci);
+      const float* Ws = Ps + net.wofs[k];       // [in][H] heads
+      const float2* Wg = net.WT2 + net.wofs[k];  // [in][H] (head, remainder)
+      const float2* bk = net.WT2 + net.bofs[k];
+      float2 s[kPtRows / 2], e[kPtRows / 2];
+      Grad<DT> gr[kPtRows];
+      int row[kPtRows];
+      // An output's value z and gradient: to the next layer's records, or to
+      // the Newton system if it is one of the zero entries.
+      auto store = [&](int x, int r, float sv, float ev, const Grad<DT>& gd) {
+        const ff z = ff_fast_two_sum(sv, ev);
+        if (x < n) {
+          float o[PS] = {z.hi, z.lo};
+#pragma unroll
+          for (int d = 0; d < DT; ++d) o[2 + d] = gd.at(d);
+#pragma unroll
+          for (int h = 0; h < PS / 4; ++h)
+            *reinterpret_cast<float4*>(next + x * PS + 4 * h) = make_float4(o[4 * h], o[4 * h + 1], o[4 * h + 2], o[4 * h + 3]);
+        } else if (x < nn) {
+#pragma unroll
+          for (int q = 0; q < DT; ++q)
+            if (zl[q] == e0 + r) {
+              gv[q] = static_cast<double>(z.hi) + static_cast<double>(z.lo);
+#pragma unroll
+              for (int d = 0; d < DT; ++d) A[q * DT + d] = gd.at(d);
+            }
+        }
+      };
+      for (int b0 = 0; b0 < nmax; b0 += kPass) {
+        const int left = nmax - b0;
+#pragma unroll
+        for (int j = 0; j < kPtRows; ++j) {
+          const int x = b0 + LN * j + gl;
+          row[j] = x < nn ? lo_[x] : 0;
+        }
+#pragma unroll
+        for (int p = 0; p < kPtRows / 2; ++p) {
+          const float2 ba = bk[row[2 * p]], bb = bk[row[2 * p + 1]];
+          s[p] = make_float2(ba.x, bb.x);
+          e[p] = make_float2(ba.y, bb.y);
+          gr[2 * p].zero();
+          gr[2 * p + 1].zero();
+        }
+        auto pass = [&](auto nr) {
+          rows_pass<DT, decltype(nr)::value, STAGED, REM>(rec, none, li, ci, cmax, Ws, Wg, row, s, e, gr);
+        };
+        switch ((left + LN - 1) / LN) {
+          case 0:
+          case 1: pass(Int<1>()); break;
+          case 2: pass(Int<2>()); break;
+          case 3: pass(Int<3>()); break;
+          case 4: pass(Int<4>()); break;
+          case 5: pass(Int<5>()); break;
+          case 6: pass(Int<6>()); break;
+          default: pass(Int<8>()); break;
+        }
+        __syncwarp();  // one pass: every input has been read (next may be rec)
+#pragma unroll
+        for (int j = 0; j < kPtRows; ++j) {
+          const int x = b0 + LN * j + gl;
+          if (x < nn) store(x, row[j], (j & 1) ? s[j >> 1].y : s[j >> 1].x, (j & 1) ? e[j >> 1].y : e[j >> 1].x, gr[j]);
+        }
+      }
+      __syncwarp();
+      // this layer's outputs are the next one's inputs
+      ci = n;
+      if (k < lall) {
+        const int Hn = net.w[k + 2];
+        for (int x = gl; x < n; x += LN) li[x] = static_cast<uint16_t>(lo_[x] * Hn);  // < 2^16
+      }
+      float* t1 = rec;
+      rec = next;
+      next = t1;
+    }
+    // the Newton step
+    float M[DT];
+#pragma unroll
+    for (int d = 0; d < DT; ++d) M[d] = 0.f;
+    float rhs = 0.f;
+    if (act && gl < DT) {
+      if (mine >= m) {
+#pragma unroll
+        for (int d = 0; d < DT; ++d) M[d] = A[gl * DT + d];
+        rhs = static_cast<float>(-gv[gl]);
+      }
+    }
+    // box facet 2d: x_d - lo_d, 2d + 1: hi_d - x_d; a polyhedral domain's facet
+    // j: c_j - A_j x; values in float64 from the stored coordinates
+    if (net.fA != nullptr) {
+      double f = 0.0;
+      const bool facet = act && gl < DT && mine < m;
+      if (facet) f = net.fc[mine];
+#pragma unroll
+      for (int d = 0; d < DT; ++d) {
+        const double x = __shfl_sync(0xffffffffu, xd, d, LN);
+        if (facet) {
+          const double a = net.fA[(long long)mine * DT + d];
+          f -= a * x;
+          M[d] = static_cast<float>(-a);
+        }
+      }
+      if (facet) rhs = static_cast<float>(-f);
+    } else {
+      const int fd = mine >> 1;
+      const double x = __shfl_sync(0xffffffffu, xd, mine < m ? fd : 0, LN);
+      if (act && gl < DT && mine < m) {
+#pragma unroll
+        for (int d = 0; d < DT; ++d)
+          if (d == fd) M[d] = (mine & 1) ? -1.f : 1.f;
+        rhs = static_cast<float>(-((mine & 1) ? (net.hi[fd] - x) : (x - net.lo[fd])));
+      }
+    }
+    bool ok = act;
+    const float dx = solve_group<DT, LN>(M, rhs, ok);
+    if (ok && gl < DT) st.X[(long long)gl * Vcap + v] = xd + static_cast<double>(dx);
+    if (ok && gl == 0) npol += 1;
+    __syncwarp();
+  }
+}
+
+// staged: the weights' heads fit in shared memory behind the vertices'
+// workspace (they are used if the network has no remainders).
+template <int DT, int LN>
+__global__ void __launch_bounds__(kPtThreads, 1) k_polish_rows(NetDesc net, State st, float thr, int mw, int TV,
+                                                               long long n_params, int staged) {
   extern __shared__ __align__(16) unsigned char sm[];
-  __shared__ int s_lmax;
   __shared__ unsigned long long s_pol;
   if (cta_stopped(st)) return;
   const Counters* last = st.cnt + net.N;
   const long long nV = last->nV_before + last->nsplit;
-  const long long Vcap = st.Vcap;
-  const int S = net.S, m = net.m;
-  const PtLayout lay = pt_layout(TV, mw, S, DT);
-  double* sA = reinterpret_cast<double*>(sm + lay.A);
-  double* sgv = reinterpret_cast<double*>(sm + lay.gv);
-  uint64_t* sig = reinterpret_cast<uint64_t*>(sm + lay.sig);  // [S][TV]
-  float* ahi = reinterpret_cast<float*>(sm + lay.ahi);        // [rows][TV]
-  float* alo = reinterpret_cast<float*>(sm + lay.alo);
-  float* J = reinterpret_cast<float*>(sm + lay.J);            // [rows][DT][TV]
-  int* zl = reinterpret_cast<int*>(sm + lay.zl);              // [TV][DT]
-  int* nzs = reinterpret_cast<int*>(sm + lay.nz);             // zeros found; -1: not polished
+  if ((long long)blockIdx.x * TV >= nV || nV > st.Vcap) return;
+  const bool heads = staged && *net.rem == 0;
+  const PtLayout lay = pt_layout(TV, mw, net.S, DT);
+  float* Ps = reinterpret_cast<float*>(sm + lay.total);
   if (threadIdx.x == 0) s_pol = 0;
-  const long long ntiles = (nV + TV - 1) / TV;
-  const int nvg = TV >> 2;
-  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const long long v0 = tile * TV;
-    if (threadIdx.x == 0) s_lmax = -1;
-    for (int i = threadIdx.x; i < S * TV; i += blockDim.x) {  // coalesced over vertices
-      const int w = i / TV, vv = i - w * TV;
-      sig[i] = v0 + vv < nV ? st.SIG[(long long)w * Vcap + v0 + vv] : 0ull;
-    }
-    __syncthreads();
-    // per vertex: its zero entries, the highest layer among them, and the
-    // coordinates (float-float) with the identity as their gradient
-    for (int vv = threadIdx.x; vv < TV; vv += blockDim.x) {
-      const long long v = v0 + vv;
-      int nz = -1, ll = -1;
-      if (v < nV && !(st.exc[v] <= thr)) {
-        nz = 0;
-        for (int w = 0; w < S; ++w) {
-          uint64_t zm = zero_mask(sig[w * TV + vv], w, net.P);
-          while (zm) {
-            const int bit = __ffsll((long long)zm) - 1;
-            if (nz < DT) zl[vv * DT + nz] = w * 32 + bit / 2;
-            ++nz;
-            zm &= zm - 1;
-          }
-        }
-        if (nz != DT) nz = -1;  // not a vertex of the generic complex: left as it is
-        for (int q = 0; nz == DT && q < DT; ++q) {
-          const int h = zl[vv * DT + q] - m;
-          if (h < 0) continue;
-          int l = 0;
-          while (l + 1 < net.L && h >= net.off[l + 1]) ++l;
-          ll = l > ll ? l : ll;
-        }
-        if (nz == DT) atomicMax(&s_lmax, ll);
-      }
-      nzs[vv] = nz;
-#pragma unroll
-      for (int d = 0; d < DT; ++d) {
-        const double x = nz == DT ? st.X[(long long)d * Vcap + v] : 0.0;
-        const float h = static_cast<float>(x);
-        ahi[d * TV + vv] = h;
-        alo[d * TV + vv] = static_cast<float>(x - static_cast<double>(h));
-#pragma unroll
-        for (int dd = 0; dd < DT; ++dd) J[(d * DT + dd) * TV + vv] = d == dd ? 1.f : 0.f;
-      }
-    }
-    __syncthreads();
-    const int lmax = s_lmax;
-    int in = DT;
-    for (int k = 0; k <= lmax; ++k) {
-      const int H = net.w[k + 1];
-      const int nrg = (H + kPtRows - 1) / kPtRows;
-      const int p = threadIdx.x;
-      const bool busy = p < nvg * nrg;
-      const int vb = busy ? (p % nvg) * 4 : 0;  // vertex blocks vary fastest in a warp
-      const int rb = busy ? (p / nvg) * kPtRows : 0;
-      // accumulators of vertex pairs (vb, vb + 1) and (vb + 2, vb + 3): the
-      // float-float arithmetic runs on packed FP32 pairs (two lanes of work
-      // per instruction, each rounded as the scalar operation)
-      float2 s2[2][kPtRows], e2[2][kPtRows], jd2[2][kPtRows][DT];
-      if (busy) {
-        const float2* Wt = net.WT2 + net.wofs[k];  // [in][H] (head, remainder)
-        const float2* bk = net.WT2 + net.bofs[k];
-#pragma unroll
-        for (int j = 0; j < kPtRows; ++j) {
-          const float2 b = rb + j < H ? bk[rb + j] : make_float2(0.f, 0.f);
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            s2[h][j] = make_float2(b.x, b.x);
-            e2[h][j] = make_float2(b.y, b.y);
-#pragma unroll
-            for (int d = 0; d < DT; ++d) jd2[h][j][d] = make_float2(0.f, 0.f);
-          }
-        }
-#pragma unroll 4
-        for (int c = 0; c < in; ++c) {
-          const float4 ah = *reinterpret_cast<const float4*>(ahi + c * TV + vb);
-          const float4 al = *reinterpret_cast<const float4*>(alo + c * TV + vb);
-          float4 jv[DT];
-#pragma unroll
-          for (int d = 0; d < DT; ++d) jv[d] = *reinterpret_cast<const float4*>(J + (c * DT + d) * TV + vb);
-          float2 w[kPtRows];
-#pragma unroll
-          for (int j = 0; j < kPtRows; ++j) w[j] = rb + j < H ? __ldg(Wt + (long long)c * H + rb + j) : make_float2(0.f, 0.f);
-          const float2 yh[2] = {make_float2(ah.x, ah.y), make_float2(ah.z, ah.w)};
-          const float2 yl[2] = {make_float2(al.x, al.y), make_float2(al.z, al.w)};
-#pragma unroll
-          for (int j = 0; j < kPtRows; ++j) {
-            const float2 xh = make_float2(w[j].x, w[j].x), xl = make_float2(w[j].y, w[j].y);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const float2 pr = __fmul2_rn(xh, yh[h]);
-              float2 er = __ffma2_rn(xh, yh[h], neg2(pr));  // exact low part of the product
-              er = __ffma2_rn(xh, yl[h], er);                // cross terms of the low parts
-              er = __ffma2_rn(xl, yh[h], er);
-              const float2 t = __fadd2_rn(s2[h][j], pr);     // TwoSum: t + its error is exact
-              const float2 bb = __fadd2_rn(t, neg2(s2[h][j]));
-              const float2 ts = __fadd2_rn(s2[h][j], neg2(__fadd2_rn(t, neg2(bb))));
-              e2[h][j] = __fadd2_rn(e2[h][j], __fadd2_rn(__fadd2_rn(ts, __fadd2_rn(pr, neg2(bb))), er));
-              s2[h][j] = t;
-            }
-#pragma unroll
-            for (int d = 0; d < DT; ++d) {
-              jd2[0][j][d] = __ffma2_rn(xh, make_float2(jv[d].x, jv[d].y), jd2[0][j][d]);
-              jd2[1][j][d] = __ffma2_rn(xh, make_float2(jv[d].z, jv[d].w), jd2[1][j][d]);
-            }
-          }
-        }
-      }
-      __syncthreads();  // every input of the layer has been read
-      if (busy) {
-#pragma unroll
-        for (int j = 0; j < kPtRows; ++j) {
-          const int r = rb + j;
-          if (r >= H) continue;
-          const int entry = m + net.off[k] + r;
-          float zh[4], zo[4], g[DT][4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float2 sp = s2[i >> 1][j], ep = e2[i >> 1][j];
-            const ff z = ff_fast_two_sum((i & 1) ? sp.y : sp.x, (i & 1) ? ep.y : ep.x);
-            zh[i] = z.hi;
-            zo[i] = z.lo;
-#pragma unroll
-            for (int d = 0; d < DT; ++d) g[d][i] = (i & 1) ? jd2[i >> 1][j][d].y : jd2[i >> 1][j][d].x;
-            const int vv = vb + i;
-            const int nz = nzs[vv];
-            for (int q = 0; q < nz; ++q)
-              if (zl[vv * DT + q] == entry) {
-                sgv[vv * DT + q] = static_cast<double>(z.hi) + static_cast<double>(z.lo);
-#pragma unroll
-                for (int d = 0; d < DT; ++d) sA[(vv * DT + q) * DT + d] = g[d][i];
-              }
-          }
-          if (k < lmax) {
-            bool act[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              act[i] = ((sig[(entry >> 5) * TV + vb + i] >> (2 * (entry & 31))) & 3ull) == kPlus;
-            *reinterpret_cast<float4*>(ahi + r * TV + vb) = make_float4(act[0] ? zh[0] : 0.f, act[1] ? zh[1] : 0.f,
-                                                                       act[2] ? zh[2] : 0.f, act[3] ? zh[3] : 0.f);
-            *reinterpret_cast<float4*>(alo + r * TV + vb) = make_float4(act[0] ? zo[0] : 0.f, act[1] ? zo[1] : 0.f,
-                                                                       act[2] ? zo[2] : 0.f, act[3] ? zo[3] : 0.f);
-#pragma unroll
-            for (int d = 0; d < DT; ++d)
-              *reinterpret_cast<float4*>(J + (r * DT + d) * TV + vb) =
-                  make_float4(act[0] ? g[d][0] : 0.f, act[1] ? g[d][1] : 0.f, act[2] ? g[d][2] : 0.f,
-                              act[3] ? g[d][3] : 0.f);
-          }
-        }
-      }
-      __syncthreads();
-      in = H;
-    }
-    for (int vv = threadIdx.x; vv < TV; vv += blockDim.x) {
-      if (nzs[vv] != DT) continue;
-      const long long v = v0 + vv;
-      int* zv = zl + vv * DT;
-      double* Av = sA + (size_t)vv * DT * DT;
-      double* gvv = sgv + (size_t)vv * DT;
-      if (DOMAIN)
-        for (int q = 0; q < DT; ++q) domain_facet_rows(net, st, v, zv, DT, q, Av, gvv);
-      NewtonOut o{};
-      newton_solve<float>(net, st, v, zv, DT, Av, gvv, o);
-      if (o.ok) {
-        for (int d = 0; d < DT; ++d) st.X[(long long)d * Vcap + v] += o.dlt[d];
-        atomicAdd(&s_pol, 1ull);
-      }
-    }
-    __syncthreads();
-  }
+  if (threadIdx.x < pt_record(DT)) reinterpret_cast<float*>(sm + lay.nz)[threadIdx.x] = 0.f;
+  if (heads)
+    for (long long t = threadIdx.x; t < n_params; t += blockDim.x) Ps[t] = net.WT2[t].x;
+  __syncthreads();
+  int npol = 0;
+  if (heads) polish_vertices<DT, LN, true>(net, st, thr, mw, TV, sm, Ps, nV, npol);
+  else polish_vertices<DT, LN, false>(net, st, thr, mw, TV, sm, Ps, nV, npol);
+  if (npol) atomicAdd(&s_pol, (unsigned long long)npol);
+  __syncthreads();
   if (threadIdx.x == 0 && s_pol) atomic_add_ll(&st.g->polished, static_cast<long long>(s_pol));
 }
 
-template <int DT>
-static cudaError_t pt_launch_d(const NetDesc& net, const State& st, float thr, int mw, int num_sms, bool domain,
+template <int DT, int LN>
+static cudaError_t pt_launch_d(const NetDesc& net, const State& st, float thr, int mw, int num_sms, long long n_params,
                                cudaStream_t stream) {
-  const int TV = pt_tile_vertices(mw, net.S, DT);
-  const size_t smem = pt_layout(TV, mw, net.S, DT).total;
-  const void* f = domain ? (const void*)k_polish_tile<DT, true> : (const void*)k_polish_tile<DT, false>;
+  int TV = pt_tile_vertices(mw, net.S, DT);
+  // the weights' heads beside at least half the vertices, or none
+  const size_t heads = (size_t)(n_params + 3) / 4 * 16;
+  const int least = std::max(4, TV / 2);
+  int tv = TV;
+  while (tv > least && pt_layout(tv, mw, net.S, DT).total + heads > (size_t)kPtSmemAll) tv -= 4;
+  const bool staged = pt_layout(tv, mw, net.S, DT).total + heads <= (size_t)kPtSmemAll;
+  if (staged) TV = tv;
+  const size_t smem = pt_layout(TV, mw, net.S, DT).total + (staged ? heads : 0);
+  const int threads = TV * LN;  // whole warps: TV is a multiple of 4
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kPtThreads, smem);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_polish_rows<DT, LN>, threads, smem);
   if (e != cudaSuccess) return e;
-  const int grid = std::max(1, num_sms * std::max(1, per_sm));  // persistent: tiles dealt round-robin
-  if (domain) k_polish_tile<DT, true><<<grid, kPtThreads, smem, stream>>>(net, st, thr, mw, TV);
-  else k_polish_tile<DT, false><<<grid, kPtThreads, smem, stream>>>(net, st, thr, mw, TV);
+  const long long tiles = (st.Vcap + TV - 1) / TV;  // persistent: vertices dealt round-robin
+  const int grid = (int)std::max<long long>(1, std::min<long long>((long long)num_sms * std::max(1, per_sm), tiles));
+  k_polish_rows<DT, LN><<<grid, threads, smem, stream>>>(net, st, thr, mw, TV, n_params, staged);
   return cudaGetLastError();
+}
+
+template <int DT>
+static cudaError_t pt_attributes() {
+  cudaError_t e = cudaFuncSetAttribute(k_polish_rows<DT, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPtSmemAll);
+  if constexpr (DT <= 8) {
+    const cudaError_t r = cudaFuncSetAttribute(k_polish_rows<DT, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPtSmemAll);
+    if (e == cudaSuccess) e = r;
+  }
+  if constexpr (DT > 1) {
+    const cudaError_t r = pt_attributes<DT - 1>();
+    if (e == cudaSuccess) e = r;
+  }
+  return e;
+}
+
+template <int DT>
+static cudaError_t pt_launch(const NetDesc& net, const State& st, float thr, int mw, int num_sms, long long n_params,
+                             cudaStream_t stream) {
+  if (net.D == DT) {
+    if constexpr (DT <= 8)
+      if (pt_lanes(mw, DT) == 8) return pt_launch_d<DT, 8>(net, st, thr, mw, num_sms, n_params, stream);
+    return pt_launch_d<DT, 16>(net, st, thr, mw, num_sms, n_params, stream);
+  }
+  if constexpr (DT > 1) return pt_launch<DT - 1>(net, st, thr, mw, num_sms, n_params, stream);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace pc
 
 using namespace pc;
 
-bool pc_polish_tile_eligible(const NetDesc& net) { return net.D >= 1 && net.D <= kPtMaxD; }
+cudaError_t pc_polish_set_attributes() { return pt_attributes<kPtMaxD>(); }
 
-cudaError_t pc_polish_tile_set_attributes() {
-  cudaError_t e = cudaSuccess;
-  auto set = [&](const void* f) {
-    const cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kPtSmemMax);
-    if (e == cudaSuccess) e = r;
-  };
-  set((const void*)k_polish_tile<1, false>);
-  set((const void*)k_polish_tile<2, false>);
-  set((const void*)k_polish_tile<3, false>);
-  set((const void*)k_polish_tile<4, false>);
-  set((const void*)k_polish_tile<5, false>);
-  set((const void*)k_polish_tile<1, true>);
-  set((const void*)k_polish_tile<2, true>);
-  set((const void*)k_polish_tile<3, true>);
-  set((const void*)k_polish_tile<4, true>);
-  set((const void*)k_polish_tile<5, true>);
-  return e;
-}
-
-cudaError_t pc_polish_tile_launch(const NetDesc& net, const State& st, float thr, int mw, int num_sms, bool domain,
-                                  cudaStream_t stream) {
-  switch (net.D) {
-    case 1: return pt_launch_d<1>(net, st, thr, mw, num_sms, domain, stream);
-    case 2: return pt_launch_d<2>(net, st, thr, mw, num_sms, domain, stream);
-    case 3: return pt_launch_d<3>(net, st, thr, mw, num_sms, domain, stream);
-    case 4: return pt_launch_d<4>(net, st, thr, mw, num_sms, domain, stream);
-    case 5: return pt_launch_d<5>(net, st, thr, mw, num_sms, domain, stream);
-    default: return cudaErrorInvalidValue;
-  }
+cudaError_t pc_polish_launch(const NetDesc& net, const State& st, float thr, int mw, int num_sms, long long n_params,
+                             cudaStream_t stream) {
+  return pt_launch<kPtMaxD>(net, st, thr, mw, num_sms, n_params, stream);
 }
