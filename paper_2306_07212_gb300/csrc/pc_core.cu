@@ -305,29 +305,37 @@ __global__ void __launch_bounds__(kBlock, 1) k_step(NetDesc net, State st, int l
   phase_step<ZT, MIXED, WORDS>(net, st, l, i, sm, reinterpret_cast<double*>(dsm + kSmemBytes), mw);
 }
 
-// The neuron loop of layer l in one cooperative launch: the layer-start
+// The neuron loop of layer l in one launch, cooperative (a grid barrier per
+// step) or one cluster (a hardware barrier per step): the layer-start
 // decisions and first edge scan (prologue = 1; a launch that resumes after a
-// capacity halt skips them) and one grid barrier per neuron step.
+// capacity halt skips them) and one barrier per neuron step.  In a cluster the
+// fatal error bits are looked at per launch only: every access is checked
+// against its bounds anyway.
 template <typename ZT, bool MIXED, int WORDS>
 __global__ void __launch_bounds__(kBlock, 1) k_layer(NetDesc net, State st, int l, int i_begin, int prologue,
-                                                     int mw) {
+                                                     int mw, int cluster) {
   extern __shared__ __align__(16) unsigned char dsm[];
   Smem& sm = *reinterpret_cast<Smem*>(dsm);
   double* ws = reinterpret_cast<double*>(dsm + kSmemBytes);
   if (cta_stopped(st)) return;
   unsigned int passed = 0;
+  auto barrier = [&]() {
+    if (!cluster) return grid_barrier(st.g, passed);
+    cluster_barrier();
+    return true;
+  };
   const int H = net.w[l + 1];
   if (threadIdx.x == 0) sm.nrl_layer = -1;
   __syncthreads();
   if (prologue) {
     phase_decide<ZT, MIXED>(net, st, l, sm, ws, mw);
-    if (!grid_barrier(st.g, passed)) return;  // uniform per CTA
+    if (!barrier()) return;  // uniform per CTA
     phase_scan0(net, st, l, sm);
-    if (!grid_barrier(st.g, passed)) return;
+    if (!barrier()) return;
   }
   for (int i = i_begin; i < H; ++i) {
     if (phase_step<ZT, MIXED, WORDS>(net, st, l, i, sm, ws, mw)) return;  // every CTA takes the same decision
-    if (i + 1 < H && !grid_barrier(st.g, passed)) return;
+    if (i + 1 < H && !barrier()) return;
   }
 }
 
@@ -588,6 +596,26 @@ struct TimerScope {
   }
 };
 
+// CTAs of a layer that runs as one cluster: 16 where the device takes that size
+// (32 splits each at a time), else the portable 8; 0: the layer does not.  A
+// step of a 2-40x4-1 net (1.8e3 vertices) takes 8.3 us in a cluster and 9.5 us
+// in the cooperative grid; of a 2-128x4-1 net (1e5) 28 and 23 us, since a
+// cluster holds fewer splits and shares one edge scan among fewer CTAs: so a
+// persistent extraction takes the cluster up to kClusterV vertices of capacity,
+// the capacity that a context starts with.  Stepwise (concurrent requests) a
+// step and neuron's launch costs about 18 us, most of it the host's with 8
+// requests at a time: up to kClusterE edges of capacity a layer is one launch of
+// one cluster there.
+constexpr long long kClusterV = 16384;
+constexpr long long kClusterE = 1ll << 20;
+
+static int cluster_ctas(const pc_ctx* c) {
+  const bool small = c->opt.exec == PC_EXEC_PERSISTENT ? c->Vcap <= kClusterV && !c->net.debug_barrier
+                                                       : c->Ecap <= kClusterE;
+  if (!small) return 0;
+  return c->big_cluster && c->Vcap > 64ll * c->N ? 16 : 8;
+}
+
 template <typename ZT, bool MIXED>
 struct Kernels {
   static void gemm(pc_ctx* c, const State& st, int l) {
@@ -609,21 +637,35 @@ struct Kernels {
   static void layer(pc_ctx* c, const State& st, int l, int i_begin, bool prologue) {
     TimerScope ts(c, 2 * l + 1);
     const int H = c->net.w[l + 1];
-    if (c->opt.exec == PC_EXEC_PERSISTENT) {
+    const auto fn = c->net.S > 16 ? k_layer<ZT, MIXED, 2> : k_layer<ZT, MIXED, 1>;
+    const int cl = cluster_ctas(c);
+    if (cl) {
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = cl;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(cl);
+      cfg.blockDim = dim3(kBlock);
+      cfg.dynamicSmemBytes = c->res_smem;
+      cfg.stream = c->stream;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      PC_CUDA(cudaLaunchKernelEx(&cfg, fn, c->net, st, l, i_begin, prologue ? 1 : 0, c->mw, 1));
+      c->launches += 1;
+    } else if (c->opt.exec == PC_EXEC_PERSISTENT) {
       PC_CUDA(cudaMemsetAsync(&static_cast<Global*>(c->g)->barrier, 0, sizeof(unsigned int), c->stream));
-      auto fn = c->net.S > 16 ? k_layer<ZT, MIXED, 2> : k_layer<ZT, MIXED, 1>;
       NetDesc net = c->net;
       State s = st;
-      int l_ = l, ib = i_begin, pro = prologue ? 1 : 0, mw = c->mw;
-      void* args[] = {&net, &s, &l_, &ib, &pro, &mw};
+      int l_ = l, ib = i_begin, pro = prologue ? 1 : 0, mw = c->mw, no = 0;
+      void* args[] = {&net, &s, &l_, &ib, &pro, &mw, &no};
       PC_CUDA(cudaLaunchCooperativeKernel((const void*)fn, dim3(c->grid_persist), dim3(kBlock), args,
                                           c->res_smem, c->stream));
       c->launches += 1;
     } else {
-      // grids sized to the edge capacity (4096 edges per CTA, which takes 32
-      // splits at a time), so that the small extractions of concurrent
-      // requests share the GPU; every phase is written for any grid size
-      const int gs = int(std::max<long long>(8, std::min<long long>(c->grid_step, c->Ecap / 4096)));
+      // grids sized to the edge capacity (8192 edges per CTA), so that
+      // concurrent requests share the GPU; every phase is written for any grid
+      const int gs = int(std::max<long long>(8, std::min<long long>(c->grid_step, c->Ecap / 8192)));
       if (prologue) {
         k_decide<ZT, MIXED><<<gs, kBlock, c->res_smem, c->stream>>>(c->net, st, l, c->mw);
         PC_CUDA(cudaGetLastError());
@@ -1075,6 +1117,12 @@ static cudaError_t set_func_attributes_now() {
   set((const void*)k_step<float, false, 2>, kSmemBytes + kRdSmemMax);
   set((const void*)k_step<float, true, 1>, kSmemBytes + kRdSmemMax);
   set((const void*)k_step<float, true, 2>, kSmemBytes + kRdSmemMax);
+  for (const void* f : {(const void*)k_layer<double, false, 1>, (const void*)k_layer<double, false, 2>,
+                        (const void*)k_layer<float, false, 1>, (const void*)k_layer<float, false, 2>,
+                        (const void*)k_layer<float, true, 1>, (const void*)k_layer<float, true, 2>}) {
+    const cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = r;
+  }
   set((const void*)k_scan0, kSmemBytes);
   {
     const cudaError_t r = pc_gemm_tc_set_attributes();
@@ -1104,6 +1152,27 @@ static cudaError_t set_func_attributes() {
   const cudaError_t e = set_func_attributes_now();
   if (e == cudaSuccess) done[dev] = true;
   return e;
+}
+
+// Whether a cluster of 16 CTAs of k_layer fits on the current device (at the
+// largest shared memory it is launched with).
+static bool big_cluster_fits() {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 16;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(16);
+  cfg.blockDim = dim3(kBlock);
+  cfg.dynamicSmemBytes = kSmemBytes + kRdSmemMax;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, k_layer<float, true, 2>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return n > 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -1146,6 +1215,7 @@ pc_status pc_create(pc_ctx** out, int device, const pc_options* opt) {
     delete c;
     return PC_ERR_CUDA;
   }
+  c->big_cluster = big_cluster_fits();
   *out = c;
   return PC_OK;
 }

@@ -66,6 +66,7 @@ struct StateBufs {
 struct pc_ctx {
   int device = 0;
   int num_sms = 1;
+  bool big_cluster = false;  // the device runs a layer in one cluster of 16 CTAs
   pc_options opt{};
   std::string err;
   cudaStream_t stream = nullptr;

@@ -217,6 +217,13 @@ __device__ __forceinline__ bool cta_stopped(const State& st) {
   return __syncthreads_or(threadIdx.x == 0 && stopped(st)) != 0;
 }
 
+// Barrier of a launch that is one cluster: in hardware, with the ordering of
+// the CTAs' global memory accesses (release / acquire).  CTAs that have
+// returned do not count, so no wait can run forever.
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // Grid-wide barrier for cooperative launches.  Bounded: after ~0.7 s of
 // polls it sets kErrTimeout and returns false (the caller then exits).  The
 // poll reads the error bits with the arrival counter (one 8-byte load), so a
