@@ -49,6 +49,7 @@ constexpr int kRankThreads = 256;
 constexpr int kTileThreads = 256;
 constexpr int kTileRounds = 16;    // items per thread of a radix tile
 constexpr int kTile = kTileThreads * kTileRounds;
+constexpr size_t kCanonKeep = 16 << 20;  // bytes of scratch a context keeps between calls
 constexpr int kGroupMax = 64;      // groups up to this size are ranked by counting
 
 // Exclusive prefix sum of counts[0..m) in place, one CTA of 1024 threads.
@@ -459,18 +460,25 @@ void pc_canonicalize(pc_ctx* c) {
   const long long vtiles = (nV + 1023) / 1024;
   // one scratch for the three phases: the sort, the rows on their way, the edges' rows
   const size_t edge_bytes = 4ull * nE + 4ull * nV + 4ull * vtiles;
-  void* perm = ctx_alloc(c, sizeof(int) * nV);
-  void* rank = ctx_alloc(c, sizeof(int) * nV);
-  void* work = ctx_alloc(c, std::max<size_t>({sort_scratch(nV), row_bytes * (size_t)nV, edge_bytes}));
-  auto release = [&]() {
-    ctx_free(c, perm);
-    ctx_free(c, rank);
-    ctx_free(c, work);
-  };
-  if (!perm || !rank || !work) {
-    release();
-    throw PcError(PC_ERR_OOM, "canonical order: device allocation failed");
+  // perm, rank and the scratch in one buffer, which a context keeps while it is
+  // small: the small results are where an allocation per call would show
+  auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+  const size_t index_bytes = up(sizeof(int) * (size_t)nV);
+  const size_t bytes = 2 * index_bytes + std::max<size_t>({sort_scratch(nV), row_bytes * (size_t)nV, edge_bytes});
+  if (c->canon_cap < bytes) {
+    ctx_free(c, c->canon_buf);
+    c->canon_buf = ctx_alloc(c, bytes);
+    c->canon_cap = c->canon_buf ? bytes : 0;
+    if (!c->canon_buf) throw PcError(PC_ERR_OOM, "canonical order: device allocation failed");
   }
+  void* perm = c->canon_buf;
+  void* rank = static_cast<char*>(perm) + index_bytes;
+  void* work = static_cast<char*>(rank) + index_bytes;
+  auto release = [&]() {
+    if (c->canon_cap <= kCanonKeep) return;
+    ctx_free(c, c->canon_buf);
+    c->canon_cap = 0;
+  };
   auto check = [&](cudaError_t e) {
     if (e != cudaSuccess) {
       release();

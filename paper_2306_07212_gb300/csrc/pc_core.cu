@@ -51,33 +51,39 @@ __global__ void k_prep(NetDesc net, float* W32, float* norms, long long n_params
     reinterpret_cast<float2*>(W32 + pairs_offset(n_params))[dst] = make_float2(h, lo);
     if (lo != 0.f) *rem = 1;  // also a NaN
   }
-  if (blockIdx.x < net.L) {
+  if (blockIdx.x < net.L) {  // one CTA per layer, one warp per neuron
     const int l = blockIdx.x, H = net.w[l + 1], K = net.w[l];
-    __shared__ double s_w[256], s_b[256];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    __shared__ double s_w[32], s_b[32];
     double mw = 0.0, mb = 0.0;
-    for (int j = threadIdx.x; j < H; j += blockDim.x) {
+    for (int j = warp; j < H; j += warps) {
       double s = 0.0;
-      for (int k = 0; k < K; ++k) {
+      for (int k = lane; k < K; k += 32) {
         const double w = net.W64[net.wofs[l] + (long long)j * K + k];
         s += w * w;
       }
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       const double bj = fabs(net.W64[net.bofs[l] + j]);
-      mw = fmax(mw, sqrt(s));
+      mw = fmax(mw, s);
       mb = fmax(mb, bj);
-      float* nr = norms + 2 * kMaxL + 3 * (net.off[l] + j);
-      nr[0] = __double2float_ru(sqrt(s) * (1.0 + 1e-6));
-      nr[1] = __double2float_ru(bj);
-      nr[2] = s > 0.0 ? __double2float_rd(1.0 / (sqrt(s) * (1.0 + 1e-6))) : 0.f;
+      if (lane == 0) {
+        float* nr = norms + 2 * kMaxL + 3 * (net.off[l] + j);
+        nr[0] = __double2float_ru(sqrt(s) * (1.0 + 1e-6));
+        nr[1] = __double2float_ru(bj);
+        nr[2] = s > 0.0 ? __double2float_rd(1.0 / (sqrt(s) * (1.0 + 1e-6))) : 0.f;
+      }
     }
-    s_w[threadIdx.x] = mw;
-    s_b[threadIdx.x] = mb;
+    if (lane == 0) {
+      s_w[warp] = mw;
+      s_b[warp] = mb;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-      for (int q = 1; q < blockDim.x; ++q) {
+      for (int q = 1; q < warps; ++q) {
         mw = fmax(mw, s_w[q]);
         mb = fmax(mb, s_b[q]);
       }
-      norms[2 * l] = __double2float_ru(mw * (1.0 + 1e-6));
+      norms[2 * l] = __double2float_ru(sqrt(mw) * (1.0 + 1e-6));
       norms[2 * l + 1] = __double2float_ru(mb);
     }
   }
@@ -412,7 +418,13 @@ static size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 void* ctx_alloc(pc_ctx* c, size_t bytes) {
   bytes = round_up(std::max<size_t>(bytes, 256), 256);
-  if (c->opt.mem_budget_bytes > 0 && c->allocated + bytes > (size_t)c->opt.mem_budget_bytes) return nullptr;
+  if (c->opt.mem_budget_bytes > 0 && c->allocated + bytes > (size_t)c->opt.mem_budget_bytes) {
+    // the kept scratch makes room first (it is not in use: the canonical order
+    // allocates nothing while it holds it)
+    ctx_free(c, c->canon_buf);
+    c->canon_cap = 0;
+    if (c->allocated + bytes > (size_t)c->opt.mem_budget_bytes) return nullptr;
+  }
   void* p = nullptr;
   if (c->alloc_fn) {
     p = c->alloc_fn(bytes, c->stream, c->alloc_user);
@@ -904,7 +916,7 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
   int* rem = reinterpret_cast<int*>(static_cast<float*>(c->norms) + 2 * kMaxL + 3 * n);
   net.rem = rem;
   PC_CUDA(cudaMemsetAsync(rem, 0, sizeof(int), c->stream));
-  k_prep<<<std::max(L, 64), 256, 0, c->stream>>>(net, static_cast<float*>(c->params32), static_cast<float*>(c->norms), p,
+  k_prep<<<std::max(L, 64), 512, 0, c->stream>>>(net, static_cast<float*>(c->params32), static_cast<float*>(c->norms), p,
                                                  rem);
   PC_CUDA(cudaGetLastError());
 
@@ -1230,6 +1242,7 @@ pc_status pc_destroy(pc_ctx* c) {
   ctx_free(c, c->cnt);
   ctx_free(c, c->g);
   ctx_free(c, c->dom_buf);
+  ctx_free(c, c->canon_buf);
   pc_poset_release(c);
   c->release_extra();
   cudaStreamSynchronize(c->stream);
@@ -1588,7 +1601,7 @@ extern "C" pc_status pc_extract_noalloc(int L, const int32_t* widths, const doub
     int* rem = reinterpret_cast<int*>(base + kNaOffNorm) + 2 * kMaxL + 3 * nn;
     net.rem = rem;
     PC_CUDA(cudaMemsetAsync(rem, 0, sizeof(int), c.stream));
-    k_prep<<<std::max(L, 64), 256, 0, c.stream>>>(net, reinterpret_cast<float*>(base + kNaOffP32),
+    k_prep<<<std::max(L, 64), 512, 0, c.stream>>>(net, reinterpret_cast<float*>(base + kNaOffP32),
                                                    reinterpret_cast<float*>(base + kNaOffNorm), p, rem);
     PC_CUDA(cudaGetLastError());
     // the scratch keeps the previous call's contents: reset what must start empty

@@ -98,6 +98,10 @@ struct pc_ctx {
   void* h_cnt = nullptr;
   void* h_g = nullptr;
 
+  // scratch of the canonical order (kept while small)
+  void* canon_buf = nullptr;
+  size_t canon_cap = 0;
+
   // polyhedral domain of the last extraction (facets and initial skeleton)
   void* dom_buf = nullptr;
   size_t dom_cap = 0;
