@@ -65,8 +65,12 @@ typedef enum {
 } pc_precision;
 
 typedef enum {
-  PC_EXEC_PERSISTENT = 0, /* one cooperative kernel per layer, grid barriers */
-  PC_EXEC_STEPWISE = 1    /* one kernel per step and neuron */
+  PC_EXEC_PERSISTENT = 0, /* one kernel per layer: cooperative with grid
+                             barriers, or one thread-block cluster while the
+                             vertex capacity is small */
+  PC_EXEC_STEPWISE = 1    /* grids that share the GPU with other requests: one
+                             cluster per layer up to 2^20 edges of capacity,
+                             else one kernel per step and neuron */
 } pc_exec;
 
 typedef enum {
@@ -134,8 +138,9 @@ typedef struct {
                              arrival more than the grid has, with a spin limit
                              of 4096 polls, so that the wait runs out and the
                              extraction returns PC_ERR_TIMEOUT; exercises the
-                             bounded-wait error path without hanging the GPU.
-                             No effect in PC_EXEC_STEPWISE (no grid barrier) */
+                             bounded-wait error path without hanging the GPU
+                             (layers then never run as a cluster).  No effect
+                             in PC_EXEC_STEPWISE (no grid barrier) */
   double filter_kappa_audit; /* PC_PREC_MIXED, 0 = off: values with
                              filter_kappa < |z| / estimate <= this are also
                              evaluated in FP64 at the exact vertex, but only
@@ -244,7 +249,8 @@ pc_status pc_stats(pc_ctx *ctx, int64_t *out, int n_neurons);
  * the interpolation formula of step (4) and the per-layer forward products of
  * step (1).  grad_x: D x nV float64 (row d at grad_x + d * nV), host or device.
  * grad_params: flat float64 array in the parameter layout, host or device;
- * overwritten.  Needs keep_tape = 1 at extraction (else PC_ERR_NO_TAPE). */
+ * overwritten.  Vertex adjoints are float64, the layer products sum float
+ * pairs (about 44 bits).  Needs keep_tape = 1 at extraction (else PC_ERR_NO_TAPE). */
 pc_status pc_backward(pc_ctx *ctx, const double *grad_x, double *grad_params, void *stream);
 
 /* k-cell counts of the last extraction's complex (Section 4.1: the k-faces
@@ -368,7 +374,7 @@ pc_status pc_server_destroy(pc_server *s);
  * callback, on real-time paths that forbid cudaMalloc because it can
  * synchronise the device, or under a fixed device-memory reservation).  The
  * paper has no counterpart: it is the same edge subdivision as pc_extract,
- * without a context, run one kernel per step.
+ * without a context, one cluster of 8 CTAs per layer.
  *
  * Inputs: widths (host, L+1), params (flat float64, host or device), box_lo /
  * box_hi (host, D), precision (pc_precision; mixed precision polishes as
@@ -383,7 +389,7 @@ pc_status pc_server_destroy(pc_server *s);
  * and SIG must be 8-byte aligned.  Otherwise the call returns PC_ERR_INVALID
  * before any device work.
  *
- * All other working memory is one static device array of about 10.6 MB
+ * All other working memory is one static device array of about 15 MB
  * inside the library, held on every GPU that loads it until the process
  * exits.  Limits: cap_v <= 16384, cap_e <= 65536, layer widths <= 32, at most
  * 512 neurons and 16384 parameters; beyond them the call returns

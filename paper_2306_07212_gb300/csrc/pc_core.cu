@@ -12,6 +12,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "pc.h"
@@ -236,32 +237,12 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
 #pragma unroll
       for (int jj = 0; jj < TJ; ++jj) acc[jj] = bs[jj];
       const ZT* row = Zin + v * K;
-      if (TRACK) {
-        for (int kk = 0; kk < K; ++kk) {
-          const ZT z = row[kk];
-          const ZT a = z > ZT(0) ? z : ZT(0);  // active iff its sign entry is +, iff its value is positive
-          a2 = fmaf(static_cast<float>(a), static_cast<float>(a), a2);
+      for (int kk = 0; kk < K; ++kk) {
+        const ZT z = row[kk];
+        const ZT a = z > ZT(0) ? z : ZT(0);  // active iff its sign entry is +, iff its value is positive
+        a2 = fmaf(static_cast<float>(a), static_cast<float>(a), a2);
 #pragma unroll
-          for (int jj = 0; jj < TJ; ++jj) acc[jj] = fma(Ws[jj][kk], a, acc[jj]);
-        }
-      } else {
-        // FP64 is bound by its rate (2 multiply-adds per clock and SM): each
-        // thread walks its vertex's active inputs only, a multiply-add with an
-        // inactive one adds an exact zero.  The lanes then read different
-        // weight columns, which shared memory serves within the time of the 16
-        // multiply-adds.  3-64x4-1 net: 2.75 -> 1.95 ms.
-        for (int k0 = 0; k0 < K; k0 += 64) {
-          uint64_t on = 0;
-          const int left = K - k0 < 64 ? K - k0 : 64;
-          for (int kk = 0; kk < left; ++kk) on |= static_cast<uint64_t>(row[k0 + kk] > ZT(0)) << kk;
-          while (on) {
-            const int kk = k0 + __ffsll((long long)on) - 1;
-            on &= on - 1;
-            const ZT a = row[kk];
-#pragma unroll
-            for (int jj = 0; jj < TJ; ++jj) acc[jj] = fma(Ws[jj][kk], a, acc[jj]);
-          }
-        }
+        for (int jj = 0; jj < TJ; ++jj) acc[jj] = fma(Ws[jj][kk], a, acc[jj]);
       }
     }
 #pragma unroll
@@ -277,6 +258,93 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
         rho = sqrtf(rho * rho + inh * inh);
       }
       st.esc[v] = rho;
+    }
+  }
+}
+
+// The product in float64 (layers after the first).  GB300's FP64 rate (2
+// multiply-adds per clock and SM) bounds it, and an inactive input adds an
+// exact zero, so it runs over each vertex's active inputs only: a CTA compacts
+// the rows of 32 vertices into lists in shared memory (coalesced, a warp per
+// row), then lane v walks vertex v's list and accumulates 16 outputs per warp.
+// The lanes read different weight columns, which shared memory serves within
+// the time of the 16 multiply-adds; they wait for the longest list of the 32
+// (about 5/8 of the inputs).  Sums keep their order.  3-64x4-1 net, whole
+// extraction: 2.75 ms over all inputs, 1.95 with a thread per vertex reading
+// its own row, 1.45 so.
+constexpr int kF64Rows = 64;  // outputs of a CTA
+constexpr int kF64Ld = 33;
+__host__ __device__ constexpr size_t f64_smem(int K) {
+  return sizeof(double) * ((size_t)kF64Rows * (K + 1) + (size_t)K * kF64Ld) + ((size_t)K * kF64Ld * 2 + 3) / 4 * 4 +
+         32 * 4;
+}
+
+__global__ void __launch_bounds__(128) k_gemm_f64(NetDesc net, State st, int l) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  if (cta_stopped(st)) return;
+  const Counters* c = st.cnt + net.off[l];
+  const long long nV = c->nV_before + c->nsplit;
+  if (nV < 0 || nV > st.Vcap) {
+    if (threadIdx.x == 0) report_corrupt(st.g, 1, l, nV, st.Vcap, 0);
+    return;
+  }
+  const int H = net.w[l + 1], K = net.w[l], j0 = blockIdx.y * kF64Rows;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double* Ws = reinterpret_cast<double*>(dsm);            // [64][K + 1]
+  double* av = Ws + kF64Rows * (K + 1);                   // [K][33] values by list position
+  uint16_t* ak = reinterpret_cast<uint16_t*>(av + K * kF64Ld);  // [K][33] their inputs
+  int* an = reinterpret_cast<int*>(dsm + f64_smem(K)) - 32;     // list lengths
+  if ((long long)blockIdx.x * 32 >= nV) return;
+  for (int t = threadIdx.x; t < kF64Rows * K; t += blockDim.x) {
+    const int jj = t / K, kk = t - jj * K, j = j0 + jj;
+    Ws[jj * (K + 1) + kk] = j < H ? net.W64[net.wofs[l] + (long long)j * K + kk] : 0.0;
+  }
+  const double* Zin = static_cast<const double*>(st.Z[l - 1]);
+  double* Zout = static_cast<double*>(st.Z[l]);
+  const int jw = 16 * warp;  // this warp's outputs
+  double bias[16];
+#pragma unroll
+  for (int jj = 0; jj < 16; ++jj) bias[jj] = j0 + jw + jj < H ? net.W64[net.bofs[l] + j0 + jw + jj] : 0.0;
+  for (long long base = (long long)blockIdx.x * 32; base < nV; base += (long long)gridDim.x * 32) {
+    __syncthreads();  // the lists of the tile before have been read (first: the weights)
+    for (int r = warp; r < 32; r += 4) {
+      const long long v = base + r;
+      int n = 0;
+      for (int k0 = 0; k0 < K; k0 += 32) {
+        const int k = k0 + lane;
+        const double z = v < nV && k < K ? Zin[v * K + k] : 0.0;
+        const bool on = z > 0.0;  // active iff its sign entry is +, iff its value is positive
+        const unsigned b = __ballot_sync(0xffffffffu, on);
+        if (on) {
+          const int at = n + __popc(b & ((1u << lane) - 1u));
+          av[at * kF64Ld + r] = z;
+          ak[at * kF64Ld + r] = static_cast<uint16_t>(k);
+        }
+        n += __popc(b);
+      }
+      if (lane == 0) an[r] = n;
+    }
+    __syncthreads();
+    if (j0 + jw < H) {
+      double acc[16];
+#pragma unroll
+      for (int jj = 0; jj < 16; ++jj) acc[jj] = bias[jj];
+      const int n = an[lane];
+      auto walk = [&](auto nj) {
+        for (int t = 0; t < n; ++t) {
+          const double a = av[t * kF64Ld + lane];
+          const double* w = Ws + jw * (K + 1) + ak[t * kF64Ld + lane];
+#pragma unroll
+          for (int jj = 0; jj < decltype(nj)::value; ++jj) acc[jj] = fma(w[jj * (K + 1)], a, acc[jj]);
+        }
+      };
+      if (H - j0 - jw <= 2) walk(std::integral_constant<int, 2>());  // an output layer
+      else walk(std::integral_constant<int, 16>());
+      const long long v = base + lane;
+      if (v < nV)
+#pragma unroll
+        for (int jj = 0; jj < 16; ++jj)
+          if (j0 + jw + jj < H) Zout[v * H + j0 + jw + jj] = acc[jj];
     }
   }
 }
@@ -639,6 +707,16 @@ struct Kernels {
       return;
     }
     const int H = c->net.w[l + 1];
+    if (sizeof(ZT) == 8 && l > 0) {
+      const size_t smem = f64_smem(c->net.w[l]);
+      const int per_sm = std::max(1, std::min(8, int(228 * 1024 / (smem + 1024))));
+      const dim3 grid(int(std::max<long long>(1, std::min<long long>((long long)c->num_sms * per_sm, (c->Vcap + 31) / 32))),
+                      (H + kF64Rows - 1) / kF64Rows);
+      k_gemm_f64<<<grid, 128, smem, c->stream>>>(c->net, st, l);
+      PC_CUDA(cudaGetLastError());
+      c->launches += 1;
+      return;
+    }
     dim3 grid(std::max(1, std::min<int>(c->num_sms * 8, int((c->Vcap + 127) / 128))), (H + 15) / 16);
     k_gemm_simt<ZT, MIXED><<<grid, 128, 0, c->stream>>>(c->net, st, l);
     PC_CUDA(cudaGetLastError());
@@ -1098,6 +1176,8 @@ void StateBufs::release(pc_ctx* c) {
 void pc_release_buffers(pc_ctx* c) {
   cudaSetDevice(c->device);
   c->bufs.release(c);
+  ctx_free(c, c->canon_buf);
+  c->canon_cap = 0;
   c->Vcap = c->Ecap = c->Tcap = 0;
   c->shape_D = c->shape_S = c->shape_H = 0;
   c->have_result = false;
@@ -1136,6 +1216,7 @@ static cudaError_t set_func_attributes_now() {
     if (e == cudaSuccess) e = r;
   }
   set((const void*)k_scan0, kSmemBytes);
+  set((const void*)k_gemm_f64, (int)f64_smem(kMaxWidth));
   {
     const cudaError_t r = pc_gemm_tc_set_attributes();
     if (e == cudaSuccess) e = r;
@@ -1384,7 +1465,14 @@ pc_status pc_values(pc_ctx* c, void* out) {
   const void* Z = pc_make_state(c).Z[L - 1];
   if (H == 1 || !out || c->nV == 0) return copy_rows(c, out, Z, zs, c->nV, c->nV, 1);
   void* rows = ctx_alloc(c, zs * H * c->nV);  // the device keeps them vertex by vertex
-  if (!rows) return c->fail(PC_ERR_OOM, "values: device allocation failed");
+  if (!rows) {  // no room for them: one strided copy per neuron
+    cudaError_t e = cudaSuccess;
+    for (int j = 0; j < H && e == cudaSuccess; ++j)
+      e = cudaMemcpy2DAsync(static_cast<char*>(out) + zs * c->nV * j, zs, static_cast<const char*>(Z) + zs * j, zs * H,
+                            zs, c->nV, cudaMemcpyDefault, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    return e == cudaSuccess ? PC_OK : c->fail(PC_ERR_CUDA, cudaGetErrorString(e));
+  }
   const int grid = int(std::min<long long>(4096, (c->nV * H + 255) / 256));
   if (zs == 8)
     k_value_rows<double><<<grid, 256, 0, c->stream>>>(static_cast<const double*>(Z), c->nV, H, static_cast<double*>(rows));
@@ -1453,8 +1541,8 @@ const char* pc_last_error(pc_ctx* c) { return c ? c->err.c_str() : "null context
 // edges, the 2-face hash table, counters and the parameter copies) lives in
 // one file-scope static device array, g_noalloc_scratch, whose size is fixed
 // at compile time.  Every GPU that loads the library holds that array until
-// the process exits.  The kernels are the same as pc_extract's, run one
-// kernel per step.
+// the process exits.  The kernels are the same as pc_extract's, a layer as one
+// cluster.
 namespace {
 
 constexpr long long kNaMaxV = 16384;        // vertices (caller capacity limit)

@@ -870,9 +870,10 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
   }
   const int D = net.D, m = net.m, S = net.S;
   const int R = D > 1 ? 2 * (D - 1) : 1;
-  // a 2-face key occurs twice, so at least kmax slots are at most half full
-  const long long kmax = total * (long long)(D - 1) * 2;
-  const long long tneed = kmax <= 64 ? 64 : 1ll << (64 - __clzll(kmax - 1));
+  // a 2-face key occurs twice, so the table is at most 2/5 full (4/5 if no face
+  // found its partner)
+  const long long kmax = total * (long long)(D - 1) * 2, tmin = kmax + kmax / 4;
+  const long long tneed = tmin <= 64 ? 64 : 1ll << (64 - __clzll(tmin - 1));
   const long long eneed = nE + total * (long long)D;
   const long long vneed = nV + total;
   const bool overV = vneed > st.Vcap || vneed >= (1ll << 31) || total * R >= (1ll << 31);
