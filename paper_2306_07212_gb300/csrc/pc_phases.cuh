@@ -39,8 +39,9 @@
 // when they are created.
 //
 // A new vertex whose value for a later neuron of the layer is within the FP32
-// filter is re-decided in FP64 by its CTA right after it is created, before
-// anything reads that sign (the round's flagged vertices of a CTA together).
+// filter is queued when it is created and re-decided in FP64 at the step's end
+// by its CTA (all its queued vertices together), before anything reads that
+// sign: its split's pairing and look-ahead wait for it.
 #pragma once
 
 #include "pc_device.cuh"

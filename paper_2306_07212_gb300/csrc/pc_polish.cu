@@ -16,18 +16,18 @@
 // 16 apart), so that an input's record (head, remainder and D gradient entries,
 // one or two 16-byte broadcasts from shared memory) serves up to 64 outputs,
 // and pairs of outputs run on packed FP32 instructions (each rounded as the
-// scalar form).  Weight heads are staged in shared memory when they fit; their remainders are read only for networks
-// that have any (NetDesc::rem).
+// scalar form).  Weight heads are staged in shared memory when they fit; their
+// remainders are read only for networks that have any (NetDesc::rem).
 //
 // The dot products follow Ogita-Rump-Oishi Dot2 (exact products by FMA, TwoSum
 // of the running sum, error terms summed in a float), about 44 bits; a skipped
-// zero input changes no bit of them, so every sum is the dense one's in its order.
+// zero input changes no bit of them, so every sum is the dense one's in its
+// order.
 //
 // Bound by FP32 issue.  Measured on GB300 against a dense product over tiles
 // of 32 vertices (D <= 5) and a dense pass of a warp per vertex (D > 5):
-// 3-64x4-1 (314k
-// vertices) 2.57 -> 0.77 ms, 5-40x4-1 (1e7) 39 -> 15.7 ms, 4-128x3-1 (212k) 3.8
-// -> 1.35 ms, 8-10x4-1 (369k) 7.7 -> 0.93 ms.
+// 3-64x4-1 (314k vertices) 2.57 -> 0.77 ms, 5-40x4-1 (1e7) 39 -> 15.7 ms,
+// 4-128x3-1 (212k) 3.8 -> 1.35 ms, 8-10x4-1 (369k) 7.7 -> 0.93 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -48,9 +48,8 @@ constexpr int kPtSmemAll = 224 * 1024;  // and the staged weights
 // Lanes of a vertex: 8 where they hold a layer's outputs in one pass and the
 // Newton system's rows (what is not the products -- lists, the solve, the few
 // outputs of the last layer -- then serves four vertices per instruction),
-// else 16.  With 16 lanes
-// throughout: 0.97 and 24.3 ms instead of 0.77 and 15.7 on the two first nets
-// above.
+// else 16.  With 16 lanes throughout: 0.97 and 24.3 ms instead of 0.77 and 15.7
+// on the two first nets above.
 __host__ __device__ constexpr int pt_lanes(int mw, int D) { return mw <= 8 * kPtRows && D <= 8 ? 8 : 16; }
 
 struct PtLayout {
@@ -253,7 +252,7 @@ struct Int {
   static constexpr int value = N;
 };
 
-// WEIGHTS: heads staged in shared memory (a network without remainders), or
+// STAGED: heads in shared memory (a network without remainders), or
 // pairs from global memory.
 template <int DT, int LN, bool STAGED>
 __device__ __forceinline__ void polish_vertices(const NetDesc& net, const State& st, float thr, int mw, int TV,

@@ -65,8 +65,9 @@ __global__ void k_mark_edge_ends(NetDesc net, State st, int l, unsigned char* us
 // FROM_Z (float64 values): the pass starts from the stored values of layer l,
 // whose rounding (2^-53 a step) is far inside the band too, and computes only
 // the layers beyond; otherwise (float32 values) it starts from the
-// coordinates.  On a pruned 3-64x4-1 extraction in float64 the
-// four passes take 1.7 ms instead of 4.8 (2.1 with inactive inputs multiplied too).
+// coordinates.  On a pruned 3-64x4-1 extraction in float64
+// the four passes take 1.7 ms instead of 4.8 (2.1 with inactive inputs
+// multiplied too).
 template <bool FROM_Z>
 __global__ void __launch_bounds__(32 * kPruneWarps) k_future_signs(NetDesc net, State st, int l, int mw, int Wf,
                                                                    const unsigned char* used, uint32_t* fut,
