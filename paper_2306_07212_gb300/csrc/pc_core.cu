@@ -383,8 +383,9 @@ __global__ void __launch_bounds__(kBlock, 1) k_step(NetDesc net, State st, int l
 // step) or one cluster (a hardware barrier per step): the layer-start
 // decisions and first edge scan (prologue = 1; a launch that resumes after a
 // capacity halt skips them) and one barrier per neuron step.  In a cluster the
-// fatal error bits are looked at per launch only: every access is checked
-// against its bounds anyway.
+// fatal error bits are looked at per launch only: an index read from memory is
+// checked before it is used, an append before it is stored, and a step whose
+// counters are outside the capacities does not run.
 template <typename ZT, bool MIXED, int WORDS>
 __global__ void __launch_bounds__(kBlock, 1) k_layer(NetDesc net, State st, int l, int i_begin, int prologue,
                                                      int mw, int cluster) {
@@ -807,6 +808,20 @@ static int occupancy_any(pc_ctx* c) {
   }
 }
 
+// Throws when a counter left its capacity.  A 2-face that occurred more than
+// twice makes more intersecting edges than the capacity check counts, which can
+// be the reason; the error is then the input's.
+static void check_corrupt(const Global& g) {
+  if (!(g.error & kErrCorrupt)) return;
+  if (g.error & kErrPairing)
+    throw PcError(PC_ERR_PAIRING, "a splitting 2-face occurred more than twice (non-generic input; error bits " +
+                                      std::to_string(g.error) + ")");
+  throw PcError(PC_ERR_CUDA, "a device counter left its capacity (internal error; check " +
+                                 std::to_string(g.diag_site) + " at " + std::to_string(g.diag_n) + ": " +
+                                 std::to_string(g.diag_a) + " " + std::to_string(g.diag_b) + " " +
+                                 std::to_string(g.diag_c) + ")");
+}
+
 // Thrown when the exact check after a fingerprint-paired extraction fails.
 struct NeedsInlinePairing {};
 
@@ -1046,11 +1061,7 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
     PC_CUDA(cudaStreamSynchronize(c->stream));
     Global g = *static_cast<Global*>(c->h_g);
     if (g.error & kErrTimeout) throw PcError(PC_ERR_TIMEOUT, "a device-side grid barrier timed out");
-    if (g.error & kErrCorrupt)
-      throw PcError(PC_ERR_CUDA, "a device counter left its capacity (internal error; check " +
-                                     std::to_string(g.diag_site) + " at " + std::to_string(g.diag_n) + ": " +
-                                     std::to_string(g.diag_a) + " " + std::to_string(g.diag_b) + " " +
-                                     std::to_string(g.diag_c) + ")");
+    check_corrupt(g);
     if (g.halted_at < 0) break;
     if (attempt > 60) throw PcError(PC_ERR_OOM, "capacity growth did not converge");
     // grow what ran out and resume at the halted neuron
@@ -1125,9 +1136,7 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
   c->nE = last.nE_before + last.nsplit + last.npairs;
   c->have_result = true;
   const Global g = *static_cast<Global*>(c->h_g);
-  if (g.error & kErrCorrupt)
-    throw PcError(PC_ERR_CUDA, "a device counter left its capacity (internal error; check " +
-                                   std::to_string(g.diag_site) + " at " + std::to_string(g.diag_n) + ")");
+  check_corrupt(g);
   if (g.error & kErrVerify) throw NeedsInlinePairing();
   long long degenerate = 0, undecided = 0;
   bool pairing = (g.error & (kErrPairing | kErrProbe)) != 0;

@@ -119,7 +119,10 @@ __device__ __forceinline__ bool step_counts(const State& st, int n, long long& n
   return nV >= 0 && nV <= st.Vcap && nE >= 0 && nE <= st.Ecap;
 }
 
+// Entry k of a list.  Each edge is listed at most once, so k < Ecap as long as
+// the step's edges fit (see pair_store for when they do not).
 __device__ __forceinline__ void list_store(int32_t* list, long long Ecap, long long k, const ListEntry& x) {
+  if (k >= Ecap) return;
   list[k] = x.e;
   list[Ecap + k] = x.p;
   list[2 * Ecap + k] = x.q;
@@ -746,10 +749,16 @@ __device__ __forceinline__ bool warp_face_matches(const State& st, long long k2,
 // ---------------------------------------------------------------------------
 // One intersecting edge to position x: its record, and its nx (listed at lb
 // + its rank among the listed ones if the next neuron crosses it).
+// The capacity check of a step counts two arrivals at a 2-face, as a generic
+// input has them.  When signs are rounding noise a 2-face can be met more often
+// and every later arrival pairs too (and raises kErrPairing), so x can pass
+// the capacity: such an edge is counted but not stored, and the next kernel
+// that reads the counters finds them above the capacity and stops.
 __device__ __forceinline__ bool pair_splits(const int4& rec) { return (rec.w ^ (rec.w >> 1)) & 1; }
 
 __device__ __forceinline__ void pair_store(const State& st, long long x, const int4& rec, int n, bool ahead,
                                            int32_t* lnext, long long at) {
+  if (x >= st.Ecap) return;
   st.EU[x] = rec.x;
   st.EW[x] = rec.y;
   if (st.deferred) st.vlist[x] = make_int4(rec.x, rec.y, rec.z, n + 1);
