@@ -81,35 +81,96 @@ __device__ inline bool solve_warp(int D, const float (&A)[kMaxD], float rhs, flo
   return true;
 }
 
-// The same step with float64 accuracy by one warp (all lanes call it; the
-// zero set has D entries): a float32 solve and two float32 corrections of its
-// residual, which is formed in float64 (iterative refinement; each one gains
-// the accuracy of a float32 solve).  A float64 division takes ~2000 clocks
-// on this chip: an elimination in float64 took 9,500 clocks at D = 3.  dl: component of the step in lane d < D.  False
-// when the system is singular.
-__device__ inline bool newton_warp(const NetDesc& net, const State& st, long long v, const int* s_zl, const double* A,
-                                   const double* gv, double& dl) {
+// Row `lane` < D of a vertex's Newton system: gradient M; returns the right-hand
+// side.  Other lanes get zeros.
+__device__ __forceinline__ double newton_row(const NetDesc& net, const State& st, long long v, const int* s_zl,
+                                             const double* A, const double* gv, double (&M)[kMaxD]) {
   const int D = net.D, m = net.m, lane = threadIdx.x & 31;
-  double M[kMaxD];
-  float F[kMaxD];
 #pragma unroll
   for (int c = 0; c < kMaxD; ++c) M[c] = 0.0;
-  double r = 0.0;
-  if (lane < D) {
-    const int j = s_zl[lane];
-    if (j < m) {
-      const int d = j >> 1;
-      const double xd = st.X[(long long)d * st.Vcap + v];
+  if (lane >= D) return 0.0;
+  const int j = s_zl[lane];
+  if (j < m) {
+    const int d = j >> 1;
+    const double xd = st.X[(long long)d * st.Vcap + v];
 #pragma unroll
-      for (int c = 0; c < kMaxD; ++c) M[c] = c == d ? ((j & 1) ? -1.0 : 1.0) : 0.0;
-      r = -((j & 1) ? (net.hi[d] - xd) : (xd - net.lo[d]));
-    } else {
-#pragma unroll
-      for (int c = 0; c < kMaxD; ++c)
-        if (c < D) M[c] = A[lane * D + c];
-      r = -gv[lane];
-    }
+    for (int c = 0; c < kMaxD; ++c) M[c] = c == d ? ((j & 1) ? -1.0 : 1.0) : 0.0;
+    return -((j & 1) ? (net.hi[d] - xd) : (xd - net.lo[d]));
   }
+#pragma unroll
+  for (int c = 0; c < kMaxD; ++c)
+    if (c < D) M[c] = A[lane * D + c];
+  return -gv[lane];
+}
+
+// The step by elimination in float64 (Gauss-Jordan, partial pivoting), for the
+// systems that float32 solves do not converge on; rare, so its registers and
+// the ~2000 clocks of each of its divisions stay out of the common path.
+// False when the system is singular or not finite.
+static __device__ __noinline__ bool newton_warp64(const NetDesc& net, const State& st, long long v, const int* s_zl,
+                                                  const double* A, const double* gv, double& dl) {
+  const int D = net.D, lane = threadIdx.x & 31;
+  double M[kMaxD];
+  double r = newton_row(net, st, v, s_zl, A, gv, M);
+  int var = -1;  // the column whose pivot this lane's row is
+  double diag = 1.0;
+#pragma unroll
+  for (int c = 0; c < kMaxD; ++c) {
+    if (c >= D) break;
+    double top = lane < D && var < 0 ? fabs(M[c]) : 0.0;
+    int piv = lane;
+    for (int o = 16; o > 0; o >>= 1) {
+      const double t = __shfl_xor_sync(0xffffffffu, top, o);
+      const int p = __shfl_xor_sync(0xffffffffu, piv, o);
+      if (t > top || (t == top && p < piv)) {
+        top = t;
+        piv = p;
+      }
+    }
+    top = __shfl_sync(0xffffffffu, top, 0);  // one answer for the warp, whatever a NaN compared to
+    piv = __shfl_sync(0xffffffffu, piv, 0);
+    if (!(top > 0.0)) return false;
+    const double pv = __shfl_sync(0xffffffffu, M[c], piv);
+    if (lane == piv) {
+      var = c;
+      diag = pv;
+    }
+    const double f = lane == piv ? 0.0 : M[c] / pv;
+#pragma unroll
+    for (int k = 0; k < kMaxD; ++k)
+      if (k > c && k < D) M[k] -= f * __shfl_sync(0xffffffffu, M[k], piv);
+    r -= f * __shfl_sync(0xffffffffu, r, piv);
+  }
+  const double mine = r / diag;
+  dl = 0.0;
+  for (int c = 0; c < D; ++c) {
+    const int src = __ffs(__ballot_sync(0xffffffffu, var == c)) - 1;
+    const double y = __shfl_sync(0xffffffffu, mine, src);
+    if (lane == c) dl = y;
+  }
+  return true;
+}
+
+// The same step by one warp (all lanes call it; the zero set has D entries) to
+// the accuracy of an elimination in float64, which took 9,500 clocks at D = 3
+// (a float64 division takes ~2000 on this chip): a float32 solve, then float32
+// corrections of its residual, which is formed in float64 (iterative
+// refinement: a correction is about rho times the one before, rho ~ condition
+// number x 2^-24).  Two corrections do for condition numbers up to a few
+// hundred: the second is then below 2^-29 of the step, and what is left, rho x
+// 2^-29, below what the elimination's own rounding leaves (condition number x
+// 2^-53).  More are made until that holds.  A system whose corrections do not
+// halve, or would take more than kNewtonSolves solves (rho above ~1/6), or that
+// is singular in float32 is eliminated in float64.  dl: component of the step
+// in lane d < D.  False when the system is singular.
+constexpr int kNewtonSolves = 12;
+
+__device__ inline bool newton_warp(const NetDesc& net, const State& st, long long v, const int* s_zl, const double* A,
+                                   const double* gv, double& dl) {
+  const int D = net.D;
+  double M[kMaxD];
+  float F[kMaxD];
+  double r = newton_row(net, st, v, s_zl, A, gv, M);
   // rows scaled by an exact power of two, so that float32 holds them
   int top = 0;
 #pragma unroll
@@ -118,16 +179,21 @@ __device__ inline bool newton_warp(const NetDesc& net, const State& st, long lon
 #pragma unroll
   for (int c = 0; c < kMaxD; ++c) F[c] = static_cast<float>(M[c] * scale);
   dl = 0.0;
-  for (int it = 0; it < 3; ++it) {
+  float first = 0.f, before = 0.f;  // the largest components of the first solve and of the last one
+  for (int it = 0; it < kNewtonSolves; ++it) {
     float x;
-    if (!solve_warp(D, F, static_cast<float>(r * scale), x)) return false;
+    if (!solve_warp(D, F, static_cast<float>(r * scale), x)) break;
     dl += static_cast<double>(x);
-    if (it == 2) break;
+    const float size = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(x))));
+    if (it == 0) first = size;
+    if (it >= 2 && size <= 0x1p-29f * first) return true;
+    if (it > 0 && !(size <= 0.5f * before)) break;  // also a NaN
+    before = size;
 #pragma unroll
     for (int c = 0; c < kMaxD; ++c)
       if (c < D) r = fma(-M[c], static_cast<double>(__shfl_sync(0xffffffffu, x, c)), r);
   }
-  return true;
+  return newton_warp64(net, st, v, s_zl, A, gv, dl);
 }
 
 // ---------------------------------------------------------------------------
