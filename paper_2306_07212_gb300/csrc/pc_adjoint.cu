@@ -20,7 +20,8 @@
 // The vertices' adjoints are float64 (the steps are bound by their launches and
 // round trips, not by arithmetic), and the layer products, which are bound by
 // the rate of multiply-adds, are sums of float pairs (Ogita-Rump-Oishi Dot2,
-// ~44 bits) on the FP32 pipes, 64 times FP64's rate.  The parameter gradient is
+// ~44 bits; activations, weights and adjoints all as pairs) on the FP32 pipes, 64
+// times FP64's rate.  The parameter gradient is
 // accumulated in float64.
 #include <cuda_runtime.h>
 
@@ -169,13 +170,16 @@ __global__ void __launch_bounds__(512) k_adj_wgrad(NetDesc net, State st, const 
 // Layer start, value part: zbar_{l-1}[v][k] = act'_k(v) sum_j W_l[j][k] zbar_l[v][j].
 // A tile's rows of zbar_l are split into float pairs once in shared memory;
 // consecutive threads take consecutive k, so weights and rows are coalesced and
-// zbar_l[v][j] is one broadcast.
+// zbar_l[v][j] is one broadcast.  A weight is a float pair too; the remainders are
+// read only for a network that has any (NetDesc::rem).
 template <typename ZT>
 __global__ void __launch_bounds__(256) k_adj_back(NetDesc net, State st, const double* zbar, double* zprev, int l,
                                                   long long nVl) {
   extern __shared__ float2 sh[];  // [kAdjTile][H]
   const int H = net.w[l + 1], K = net.w[l];
   const float* W = net.W32 + net.wofs[l];
+  const float* R = net.R32 + net.wofs[l];
+  const bool pairs = *net.rem != 0;
   const ZT* Zin = static_cast<const ZT*>(st.Z[l - 1]);
   for (long long base = (long long)blockIdx.x * kAdjTile; base < nVl; base += (long long)gridDim.x * kAdjTile) {
     const int n = nVl - base < kAdjTile ? int(nVl - base) : kAdjTile;
@@ -184,8 +188,13 @@ __global__ void __launch_bounds__(256) k_adj_back(NetDesc net, State st, const d
     for (int t = threadIdx.x; t < n * K; t += blockDim.x) {
       const int c = t / K, k = t - c * K;
       float s = 0.f, e = 0.f;
-      if (Zin[base * K + t] > ZT(0))  // active iff its sign entry is +
-        for (int j = 0; j < H; ++j) dot2(sh[c * H + j], make_float2(W[(long long)j * K + k], 0.f), s, e);
+      if (Zin[base * K + t] > ZT(0)) {  // active iff its sign entry is +
+        if (pairs)
+          for (int j = 0; j < H; ++j)
+            dot2(sh[c * H + j], make_float2(W[(long long)j * K + k], R[(long long)j * K + k]), s, e);
+        else
+          for (int j = 0; j < H; ++j) dot2(sh[c * H + j], make_float2(W[(long long)j * K + k], 0.f), s, e);
+      }
       zprev[base * K + t] = static_cast<double>(s) + static_cast<double>(e);
     }
     __syncthreads();

@@ -32,7 +32,8 @@ __host__ __device__ inline long long pairs_offset(long long n_params) { return (
 // estimate: per layer max_j ||W_j||_2 and max_j |b_j|, per neuron ||W_n||_2,
 // |b_n| and 1/||W_n||_2 (rounded outward).
 // *rem (0 at the launch) becomes nonzero if any parameter is not a float32.
-__global__ void k_prep(NetDesc net, float* W32, float* norms, long long n_params, int* rem) {
+// R32 (may be null): the remainders in the parameters' order.
+__global__ void k_prep(NetDesc net, float* W32, float* R32, float* norms, long long n_params, int* rem) {
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n_params;
        t += (long long)gridDim.x * blockDim.x)
   {
@@ -50,6 +51,7 @@ __global__ void k_prep(NetDesc net, float* W32, float* norms, long long n_params
     }
     const float lo = static_cast<float>(w - static_cast<double>(h));
     reinterpret_cast<float2*>(W32 + pairs_offset(n_params))[dst] = make_float2(h, lo);
+    if (R32) R32[t] = lo;
     if (lo != 0.f) *rem = 1;  // also a NaN
   }
   if (blockIdx.x < net.L) {  // one CTA per layer, one warp per neuron
@@ -989,7 +991,8 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
     ctx_free(c, c->params32);
     ctx_free(c, c->norms);
     c->params64 = ctx_alloc(c, pbytes);
-    c->params32 = ctx_alloc(c, sizeof(float) * (pairs_offset(p) + 2 * p));  // heads, then (head, remainder) pairs
+    // heads, (head, remainder) pairs, and for the adjoint the remainders
+    c->params32 = ctx_alloc(c, sizeof(float) * (pairs_offset(p) + 2 * p + (c->opt.keep_tape ? p : 0)));
     c->norms = ctx_alloc(c, sizeof(float) * (2 * kMaxL + 3 * (size_t)n + 1));  // and the remainder flag
     if (!c->params64 || !c->params32 || !c->norms) {
       ctx_free(c, c->params64);
@@ -1009,8 +1012,10 @@ static void run_extract(pc_ctx* c, int L, const int32_t* widths, const double* p
   int* rem = reinterpret_cast<int*>(static_cast<float*>(c->norms) + 2 * kMaxL + 3 * n);
   net.rem = rem;
   PC_CUDA(cudaMemsetAsync(rem, 0, sizeof(int), c->stream));
-  k_prep<<<std::max(L, 64), 512, 0, c->stream>>>(net, static_cast<float*>(c->params32), static_cast<float*>(c->norms), p,
-                                                 rem);
+  float* R32 = c->opt.keep_tape ? static_cast<float*>(c->params32) + pairs_offset(p) + 2 * p : nullptr;
+  net.R32 = R32;
+  k_prep<<<std::max(L, 64), 512, 0, c->stream>>>(net, static_cast<float*>(c->params32), R32,
+                                                 static_cast<float*>(c->norms), p, rem);
   PC_CUDA(cudaGetLastError());
 
   // state buffers (kept across extractions when shapes allow)
@@ -1698,7 +1703,7 @@ extern "C" pc_status pc_extract_noalloc(int L, const int32_t* widths, const doub
     int* rem = reinterpret_cast<int*>(base + kNaOffNorm) + 2 * kMaxL + 3 * nn;
     net.rem = rem;
     PC_CUDA(cudaMemsetAsync(rem, 0, sizeof(int), c.stream));
-    k_prep<<<std::max(L, 64), 512, 0, c.stream>>>(net, reinterpret_cast<float*>(base + kNaOffP32),
+    k_prep<<<std::max(L, 64), 512, 0, c.stream>>>(net, reinterpret_cast<float*>(base + kNaOffP32), nullptr,
                                                    reinterpret_cast<float*>(base + kNaOffNorm), p, rem);
     PC_CUDA(cudaGetLastError());
     // the scratch keeps the previous call's contents: reset what must start empty

@@ -75,6 +75,7 @@ struct NetDesc {
   const float* W32;      // flat parameters rounded to float32
   const float2* WT2;     // per layer W^T (k-major: [K][H]) then b, as (float32 head,
                          // float32 of the remainder): about 48 bits per parameter
+  const float* R32;      // flat remainders (float32 of parameter - W32); kept with the tape only, else null
   const int* rem;        // device flag: some parameter has a remainder (is not a float32)
   const float* norms;    // per layer: [2l] = max_j ||W_j||_2, [2l+1] = max_j |b_j|
   const float* nrm;      // per neuron n: [3n] = ||W_n||_2, [3n+1] = |b_n|, [3n+2] = 1/||W_n||_2
