@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(512) k_adj_wgrad(NetDesc net, State st, const 
           val = st.X[(long long)k * Vcap + base + c];
         } else {
           const ZT z = Zin[base * K + t];
-          val = z > ZT(0) ? static_cast<double>(z) : 0.0;  // active iff its sign entry is +
+          val = z <= ZT(0) ? 0.0 : static_cast<double>(z);  // active iff its sign entry is +
         }
       }
       at[k * LD + c] = split_pair(val);
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(256) k_adj_back(NetDesc net, State st, const d
     for (int t = threadIdx.x; t < n * K; t += blockDim.x) {
       const int c = t / K, k = t - c * K;
       float s = 0.f, e = 0.f;
-      if (Zin[base * K + t] > ZT(0)) {  // active iff its sign entry is +
+      if (!(Zin[base * K + t] <= ZT(0))) {  // active iff its sign entry is +
         if (pairs)
           for (int j = 0; j < H; ++j)
             dot2(sh[c * H + j], make_float2(W[(long long)j * K + k], R[(long long)j * K + k]), s, e);

@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
       const ZT* row = Zin + v * K;
       for (int kk = 0; kk < K; ++kk) {
         const ZT z = row[kk];
-        const ZT a = z > ZT(0) ? z : ZT(0);  // active iff its sign entry is +, iff its value is positive
+        const ZT a = z <= ZT(0) ? ZT(0) : z;  // active iff its sign entry is +, iff its value is not <= 0
         a2 = fmaf(static_cast<float>(a), static_cast<float>(a), a2);
 #pragma unroll
         for (int jj = 0; jj < TJ; ++jj) acc[jj] = fma(Ws[jj][kk], a, acc[jj]);
@@ -314,8 +314,8 @@ __global__ void __launch_bounds__(128) k_gemm_f64(NetDesc net, State st, int l) 
       int n = 0;
       for (int k0 = 0; k0 < K; k0 += 32) {
         const int k = k0 + lane;
-        const double z = v < nV && k < K ? Zin[v * K + k] : 0.0;
-        const bool on = z > 0.0;  // active iff its sign entry is +, iff its value is positive
+        const double z = v < nV && k < K ? Zin[v * K + k] : 0.0;  // (a NaN's entry is +: it spreads)
+        const bool on = !(z <= 0.0);  // active iff its sign entry is +, iff its value is not <= 0
         const unsigned b = __ballot_sync(0xffffffffu, on);
         if (on) {
           const int at = n + __popc(b & ((1u << lane) - 1u));

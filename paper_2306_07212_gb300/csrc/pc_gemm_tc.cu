@@ -19,7 +19,7 @@
 // 16-byte groups of row r are permuted by XOR with r mod 8; 8-row groups are
 // 1024 B apart.  The pieces of W_l are split from FP64 and staged once per
 // CTA.  Activation chunks are gathered from the vertices' value rows (16-byte
-// loads where the rows allow; a value is positive iff its sign entry is +) and
+// loads where the rows allow; an entry is + iff the value is not <= 0) and
 // split in registers by the 128 threads (one vertex each); each piece goes to one of two
 // shared-memory buffers, so the next piece is written while the MMAs of the
 // previous one run.  One elected thread issues the MMAs and commits them to
@@ -135,8 +135,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
   for (int q = 0; q < 16; ++q) r[q] = __uint_as_float(u[q]);
 }
 
-// The vertex's 32 inputs of chunk q: its row's values where positive (a value
-// is positive iff its sign entry is +), else 0.  16-byte loads when the rows
+// The vertex's 32 inputs of chunk q: its row's values where not <= 0, else 0 (a
+// value's sign entry is + iff it is not <= 0; a NaN's is +, and it spreads).  16-byte loads when the rows
 // are 16-byte aligned.
 __device__ __forceinline__ void gather_chunk(const float* Zin, long long v, bool valid, int q, int K,
                                              float (&x)[kTcChunkK]) {
@@ -156,7 +156,7 @@ __device__ __forceinline__ void gather_chunk(const float* Zin, long long v, bool
     for (int k = 0; k < kTcChunkK; ++k) x[k] = k < left ? row[k] : 0.f;
   }
 #pragma unroll
-  for (int k = 0; k < kTcChunkK; ++k) x[k] = x[k] > 0.f ? x[k] : 0.f;
+  for (int k = 0; k < kTcChunkK; ++k) x[k] = x[k] <= 0.f ? 0.f : x[k];
 }
 
 // 16 outputs of a vertex's row, from neuron j0 (+ b_l).

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(32 * kPruneWarps) k_future_signs(NetDesc net, 
       const int r = r0 + lane;
       double x = 0.0;
       if (r < H) x = FROM_Z ? static_cast<const double*>(st.Z[l])[v * H + r] : st.X[(long long)r * Vcap + v];
-      const bool act = r < H && (!FROM_Z || x > 0.0);
+      const bool act = r < H && (!FROM_Z || !(x <= 0.0));  // a layer's value: iff its sign entry is +
       const unsigned b = __ballot_sync(0xffffffffu, act);
       if (act) {
         const int at = n + __popc(b & ((1u << lane) - 1u));
