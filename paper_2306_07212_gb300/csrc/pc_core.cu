@@ -571,7 +571,7 @@ static void realloc_state(pc_ctx* c, long long V, long long E, long long T, bool
   if (copy && ob.X) {
     const long long oV = c->Vcap, oE = c->Ecap, nV = std::min(oV, V), nE = std::min(oE, E);
     auto cp2 = [&](void* dst, size_t dpitch, const void* src, size_t spitch, size_t width, size_t rows) {
-      if (rows && width) PC_CUDA(cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows, cudaMemcpyDeviceToDevice, c->stream));
+      PC_CUDA(pc_copy_rows_async(dst, dpitch, src, spitch, width, rows, c->stream));
     };
     cp2(nb.X, 8 * V, ob.X, 8 * oV, 8 * nV, D);
     for (int k = 0; k < nb.nz && k < ob.nz; ++k) cp2(nb.Z[k], zs * Hm * V, ob.Z[k], zs * Hm * oV, zs * Hm * nV, 1);
@@ -1441,7 +1441,7 @@ pc_status pc_counts(pc_ctx* c, int64_t* nv, int64_t* ne, int32_t* sw, int32_t* d
 
 static pc_status copy_rows(pc_ctx* c, void* out, const void* src, size_t elt, long long ld, long long n, int rows) {
   if (!out || n == 0 || rows == 0) return PC_OK;
-  cudaError_t e = cudaMemcpy2DAsync(out, elt * n, src, elt * ld, elt * n, rows, cudaMemcpyDefault, c->stream);
+  cudaError_t e = pc_copy_rows_async(out, elt * n, src, elt * ld, elt * n, rows, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return c->fail(PC_ERR_CUDA, cudaGetErrorString(e));
   return PC_OK;

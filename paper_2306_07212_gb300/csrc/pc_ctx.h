@@ -40,6 +40,23 @@ cudaError_t pc_polish_set_attributes();
 cudaError_t pc_polish_launch(const pc::NetDesc& net, const pc::State& st, float thr, int mw, int num_sms,
                              long long n_params, cudaStream_t stream);
 
+// rows rows of width bytes, dpitch / spitch bytes apart, on a stream.
+// cudaMemcpy2DAsync takes pitches up to 2^31 - 1 bytes: one row has none, and
+// rows further apart are copied one by one.
+inline cudaError_t pc_copy_rows_async(void* dst, size_t dpitch, const void* src, size_t spitch, size_t width,
+                                      size_t rows, cudaStream_t stream) {
+  constexpr size_t kMaxPitch = 0x7fffffff;
+  if (rows == 0 || width == 0) return cudaSuccess;
+  if (rows > 1 && dpitch <= kMaxPitch && spitch <= kMaxPitch)
+    return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows, cudaMemcpyDefault, stream);
+  for (size_t r = 0; r < rows; ++r) {
+    const cudaError_t e = cudaMemcpyAsync(static_cast<char*>(dst) + r * dpitch, static_cast<const char*>(src) + r * spitch,
+                                          width, cudaMemcpyDefault, stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 struct PcError : std::runtime_error {
   pc_status status;
   PcError(pc_status s, const std::string& m) : std::runtime_error(m), status(s) {}
