@@ -68,9 +68,11 @@ typedef enum {
   PC_EXEC_PERSISTENT = 0, /* one kernel per layer: cooperative with grid
                              barriers, or one thread-block cluster while the
                              vertex capacity is small */
-  PC_EXEC_STEPWISE = 1    /* grids that share the GPU with other requests: one
-                             cluster per layer up to 2^20 edges of capacity,
-                             else one kernel per step and neuron */
+  PC_EXEC_STEPWISE = 1    /* no grid barrier, so that requests can share the
+                             GPU: one cluster per layer (beside other requests
+                             of a server up to 2^20 edges of capacity, alone up
+                             to 32768 vertices), else one kernel per step and
+                             neuron */
 } pc_exec;
 
 typedef enum {

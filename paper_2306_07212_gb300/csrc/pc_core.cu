@@ -685,16 +685,34 @@ struct TimerScope {
 // in the cooperative grid; of a 2-128x4-1 net (1e5) 28 and 23 us, since a
 // cluster holds fewer splits and shares one edge scan among fewer CTAs: so a
 // persistent extraction takes the cluster up to kClusterV vertices of capacity,
-// the capacity that a context starts with.  Stepwise (concurrent requests) a
-// step and neuron's launch costs about 18 us, most of it the host's with 8
-// requests at a time: up to kClusterE edges of capacity a layer is one launch of
-// one cluster there.
+// the capacity that a context starts with.
+// Stepwise the alternative is a launch per step and neuron.  Beside other
+// requests of a server it costs about 18 us, most of it the host's with 8 at a
+// time, so a layer is one cluster up to kClusterE edges of capacity: 16 requests
+// of up to 2e5 vertices take 18.5 ms, and 26 with the line at 2^18.  Alone the
+// whole chip is free for a grid, and the line is kAloneV vertices, expected or
+// of capacity: a 2-64x4-1 net (3.2e4 vertices) takes 5.4 ms in clusters and 5.8
+// in grids, a 3-20x4-1 net (7.5e4) 2.8 and 2.0, a 4-12x4-1 net (2.1e5) 4.8 and
+// 2.0.
 constexpr long long kClusterV = 16384;
 constexpr long long kClusterE = 1ll << 20;
+constexpr long long kAloneV = 32768;
+
+static bool shares_gpu(const pc_ctx* c) { return c->load && c->load->load(std::memory_order_relaxed) > 1; }
+
+// Vertices of a generic complex on a box, at most (see pc_estimate_bytes): a
+// context may hold more capacity from an earlier network.
+static double most_vertices(const NetDesc& net) {
+  double v = 1.2;
+  for (int d = 1; d <= net.D; ++d) v *= double(net.N) / d;
+  return v + std::ldexp(1.0, net.D);
+}
 
 static int cluster_ctas(const pc_ctx* c) {
-  const bool small = c->opt.exec == PC_EXEC_PERSISTENT ? c->Vcap <= kClusterV && !c->net.debug_barrier
-                                                       : c->Ecap <= kClusterE;
+  bool small;
+  if (c->opt.exec == PC_EXEC_PERSISTENT) small = c->Vcap <= kClusterV && !c->net.debug_barrier;
+  else if (shares_gpu(c) || c->Ecap > kClusterE) small = c->Ecap <= kClusterE;
+  else small = (c->net.fA ? double(c->Vcap) : std::min(double(c->Vcap), most_vertices(c->net))) <= double(kAloneV);
   if (!small) return 0;
   return c->big_cluster && c->Vcap > 64ll * c->N ? 16 : 8;
 }
@@ -756,9 +774,11 @@ struct Kernels {
                                           c->res_smem, c->stream));
       c->launches += 1;
     } else {
-      // grids sized to the edge capacity (8192 edges per CTA), so that
-      // concurrent requests share the GPU; every phase is written for any grid
-      const int gs = int(std::max<long long>(8, std::min<long long>(c->grid_step, c->Ecap / 8192)));
+      // grids sized to the edge capacity; every phase is written for any grid.
+      // 8192 edges per CTA beside other requests, so that they share the GPU; 2048
+      // alone (3-16x4-1 net, 4.3e4 vertices: 1.60 ms, and 1.90 with 8192; with
+      // 1024 within 5 % of 2048 from 3e4 vertices up)
+      const int gs = int(std::max<long long>(8, std::min<long long>(c->grid_step, c->Ecap / (shares_gpu(c) ? 8192 : 2048))));
       if (prologue) {
         k_decide<ZT, MIXED><<<gs, kBlock, c->res_smem, c->stream>>>(c->net, st, l, c->mw);
         PC_CUDA(cudaGetLastError());
@@ -1198,6 +1218,8 @@ void pc_release_buffers(pc_ctx* c) {
   pc_poset_release(c);
   cudaStreamSynchronize(c->stream);
 }
+
+void pc_set_load(pc_ctx* c, const std::atomic<int>* load) { c->load = load; }
 
 // Dynamic shared-memory limits of the kernels, set to constant maxima so that
 // every context (in any thread) agrees; a per-network value would race.

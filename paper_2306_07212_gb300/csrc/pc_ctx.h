@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstddef>
 #include <stdexcept>
 #include <string>
@@ -17,6 +18,9 @@ struct pc_ctx;
 void* ctx_alloc(pc_ctx* c, size_t bytes);
 void ctx_free(pc_ctx* c, void*& p);
 pc::State pc_make_state(pc_ctx* c);
+
+// a server's context: its count of unfinished requests
+void pc_set_load(pc_ctx* c, const std::atomic<int>* load);
 
 // canonical output order (pc_canon.cu)
 void pc_canonicalize(pc_ctx* c);
@@ -84,6 +88,7 @@ struct pc_ctx {
   int device = 0;
   int num_sms = 1;
   bool big_cluster = false;  // the device runs a layer in one cluster of 16 CTAs
+  const std::atomic<int>* load = nullptr;  // a server's requests, running or queued (null: none but this context's)
   pc_options opt{};
   std::string err;
   cudaStream_t stream = nullptr;

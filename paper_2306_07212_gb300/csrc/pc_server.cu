@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <condition_variable>
@@ -32,6 +33,9 @@
 // Frees a context's extraction buffers (pc_core.cu); the next extraction
 // allocates them again.
 void pc_release_buffers(pc_ctx* c);
+// The count of requests by which an extraction chooses between the whole GPU and
+// a share of it (pc_core.cu).
+void pc_set_load(pc_ctx* c, const std::atomic<int>* load);
 
 namespace {
 
@@ -66,7 +70,8 @@ struct pc_server {
   std::map<uint64_t, std::unique_ptr<Request>> all;
   uint64_t next_id = 1;
   int64_t in_use = 0, peak_in_use = 0;
-  int running = 0, pending = 0;
+  int running = 0;
+  std::atomic<int> pending{0};  // queued or running (written under mu)
   bool stop = false;
   std::vector<std::thread> workers;
   std::vector<pc_ctx*> ctxs;              // one extraction context per slot
@@ -217,6 +222,7 @@ pc_status pc_server_create(pc_server** out, int device, const pc_server_options*
       delete s;
       return PC_ERR_CUDA;
     }
+    pc_set_load(ctx, &s->pending);
     s->ctxs.push_back(ctx);
     s->streams.push_back(st);
   }
