@@ -52,6 +52,13 @@ __global__ void k_mark_edge_ends(NetDesc net, State st, int l, unsigned char* us
   }
 }
 
+// The polish's threshold input for the copy of the coordinates that the signs are
+// taken at: above 0 for the vertices that have an edge and a coordinate error.
+__global__ void k_polish_marks(const unsigned char* used, const float* exc, long long V, float* mark) {
+  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x)
+    mark[v] = used[v] && exc[v] != 0.f ? 1.f : 0.f;
+}
+
 // Forward pass of vertex v (one per warp) through the rest of the net, for
 // the vertices that still have an edge (used; the others are never read),
 // in float-float arithmetic (Dot2 as in the polish: exact products by FMA,
@@ -65,7 +72,8 @@ __global__ void k_mark_edge_ends(NetDesc net, State st, int l, unsigned char* us
 // FROM_Z (float64 values): the pass starts from the stored values of layer l,
 // whose rounding (2^-53 a step) is far inside the band too, and computes only
 // the layers beyond; otherwise (float32 values) it starts from the
-// coordinates.  On a pruned 3-64x4-1 extraction in float64
+// coordinates: in mixed precision, whose later signs are those at the exact
+// vertex, from polished ones (pc_prune_edges).  On a pruned 3-64x4-1 extraction in float64
 // the four passes take 1.7 ms instead of 4.8 (2.1 with inactive inputs
 // multiplied too).
 template <bool FROM_Z>
@@ -339,14 +347,13 @@ void pc_prune_edges(pc_ctx* c, const State& st, int l) {
   const int Wf = (nf + 31) / 32;
   const long long V = c->Vcap, E = c->Ecap;
   const int nblocks = static_cast<int>((E + kCompactBlock - 1) / kCompactBlock);
+  const bool newton = net.precision == PC_PREC_MIXED;
   void* fut = ctx_alloc(c, sizeof(uint32_t) * Wf * V);
   void* unc = ctx_alloc(c, V);
   void* used = ctx_alloc(c, V);
-  void* keep = ctx_alloc(c, sizeof(int) * E);
-  void* counts = ctx_alloc(c, sizeof(int) * (nblocks + 1));
-  void* tU = ctx_alloc(c, sizeof(int32_t) * E);
-  void* tW = ctx_alloc(c, sizeof(int32_t) * E);
-  void* tL = c->deferred ? ctx_alloc(c, sizeof(int4) * E) : nullptr;
+  void* px = newton ? ctx_alloc(c, sizeof(double) * net.D * V) : nullptr;
+  void* mark = newton ? ctx_alloc(c, sizeof(float) * V) : nullptr;
+  void *keep = nullptr, *counts = nullptr, *tU = nullptr, *tW = nullptr, *tL = nullptr;
   auto release = [&]() {
     ctx_free(c, fut);
     ctx_free(c, unc);
@@ -356,20 +363,54 @@ void pc_prune_edges(pc_ctx* c, const State& st, int l) {
     ctx_free(c, tU);
     ctx_free(c, tW);
     ctx_free(c, tL);
+    ctx_free(c, px);
+    ctx_free(c, mark);
   };
-  if (!fut || !unc || !used || !keep || !counts || !tU || !tW || (c->deferred && !tL)) {
+  auto refuse = [&]() {
     release();
     throw PcError(PC_ERR_OOM, "pruning: device allocation failed");
-  }
+  };
+  if (!fut || !unc || !used || (newton && (!px || !mark))) refuse();
   cudaStream_t s = c->stream;
   Counters* cn = st.cnt + net.off[l + 1];
   const size_t smem = sizeof(double) * kPruneWarps * (3 * c->mw + Wf);
   const int vgrid = static_cast<int>(std::max<long long>(1, std::min<long long>(4ll * c->num_sms, (V + kPruneWarps - 1) / kPruneWarps)));
   cudaMemsetAsync(used, 0, V, s);
   k_mark_edge_ends<<<grid_of(E), 256, 0, s>>>(net, st, l, static_cast<unsigned char*>(used));
+  // In mixed precision a later layer decides its signs at the exact vertices (to
+  // 1e-12), while the stored coordinates carry float32 errors of their crossing
+  // parameters (1e-8 of the box, more where the crossing is flat): an edge could
+  // be dropped by a sign that its vertex does not have, and its 2-faces then lose
+  // a crossing.  So the signs are taken at a polished copy of the coordinates (of
+  // the vertices that have an edge; by the layers so far).
+  State at = st;
+  cudaError_t pe = cudaSuccess;
+  if (newton) {
+    at.X = static_cast<double*>(px);
+    at.exc = static_cast<float*>(mark);
+    cudaMemcpyAsync(px, st.X, sizeof(double) * net.D * V, cudaMemcpyDeviceToDevice, s);
+    k_polish_marks<<<grid_of(V), 256, 0, s>>>(static_cast<const unsigned char*>(used), st.exc, V,
+                                              static_cast<float*>(mark));
+    NetDesc upto = net;
+    upto.L = l + 1;
+    upto.N = net.off[l + 1];
+    upto.P = net.m + upto.N;
+    pe = pc_polish_launch(upto, at, 0.f, c->mw, c->num_sms, net.wofs[l + 1], s);
+    cudaMemsetAsync(&st.g->polished, 0, sizeof(st.g->polished), s);  // counts the result's vertices only
+    c->launches += 2;
+  }
   const auto future = net.precision == PC_PREC_FP64 ? k_future_signs<true> : k_future_signs<false>;
-  future<<<vgrid, 32 * kPruneWarps, smem, s>>>(net, st, l, c->mw, Wf, static_cast<const unsigned char*>(used),
+  future<<<vgrid, 32 * kPruneWarps, smem, s>>>(net, at, l, c->mw, Wf, static_cast<const unsigned char*>(used),
                                                static_cast<uint32_t*>(fut), static_cast<unsigned char*>(unc));
+  // the edges' temporaries take the place of the coordinates' (freed in stream order)
+  ctx_free(c, px);
+  ctx_free(c, mark);
+  keep = ctx_alloc(c, sizeof(int) * E);
+  counts = ctx_alloc(c, sizeof(int) * (nblocks + 1));
+  tU = ctx_alloc(c, sizeof(int32_t) * E);
+  tW = ctx_alloc(c, sizeof(int32_t) * E);
+  tL = c->deferred ? ctx_alloc(c, sizeof(int4) * E) : nullptr;
+  if (!keep || !counts || !tU || !tW || (c->deferred && !tL)) refuse();
   k_edge_keep<<<grid_of(E), 256, 0, s>>>(net, st, l, Wf, static_cast<const uint32_t*>(fut),
                                          static_cast<const unsigned char*>(unc), static_cast<int*>(keep));
   k_block_count<<<nblocks, kCompactBlock, 0, s>>>(st.g, static_cast<const int*>(keep), nullptr, cn, 0,
@@ -381,7 +422,7 @@ void pc_prune_edges(pc_ctx* c, const State& st, int l) {
   k_edge_commit<<<grid_of(E), 256, 0, s>>>(st, cn, static_cast<const int*>(counts) + nblocks,
                                            static_cast<const int32_t*>(tU), static_cast<const int32_t*>(tW),
                                            static_cast<const int4*>(tL));
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t le = cudaGetLastError(), e = pe != cudaSuccess ? pe : le;
   release();
   if (e != cudaSuccess) throw PcError(PC_ERR_CUDA, std::string("pruning: ") + cudaGetErrorString(e));
   c->launches += 7;
