@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
       }
 #pragma unroll
       for (int jj = 0; jj < TJ; ++jj) acc[jj] = static_cast<ZT>(dacc[jj]);
-    } else {
+    } else if constexpr (sizeof(ZT) == 4) {  // float64's later layers: k_gemm_f64
 #pragma unroll
       for (int jj = 0; jj < TJ; ++jj) acc[jj] = bs[jj];
       const ZT* row = Zin + v * K;

@@ -77,7 +77,6 @@ struct Smem {
   int4 pairs[kWarps][kPairCap];        // (v_a, v_b, zero ordinals, signs at the next neuron: bit 0 v_a -, bit 1 v_b -)
   ListEntry la[kWarps][kLaCap];        // the warps' list entries for the next neuron
   int lac[kWarps], pc[kWarps], pla[kWarps];
-  int cursor;
   int npend;
   int tile;                            // next scan tile of this CTA
   long long pbase, lbase;
@@ -213,7 +212,7 @@ __host__ __device__ inline RdLayout rd_layout(int P, int mw, int D, int S) {
   r.A = take((size_t)P * D * D * 8);    // Newton rows [P][D][D]
   r.gv = take((size_t)P * D * 8);       // their values [P][D]
   r.dlt = take((size_t)P * D * 8);      // Newton steps [P][D]
-  r.sig = take((size_t)P * S * 8);      // sign words [P][S]
+  r.sig = take(0);                      // sign words: none, they become the lists below
   r.J = take((size_t)P * mw * D * 4);   // gradients (float) [P][mw][D], by list position
   r.Jn = take((size_t)P * mw * D * 4);
   r.sc = take((size_t)P * mw * 4);      // sums of |terms| of layer l [P][mw]
@@ -249,7 +248,6 @@ __device__ __noinline__ void redecide_batch(const NetDesc& net, const State& st,
   double* A = reinterpret_cast<double*>(ws + L.A);
   double* gv = reinterpret_cast<double*>(ws + L.gv);
   double* dlt = reinterpret_cast<double*>(ws + L.dlt);
-  uint64_t* sig = reinterpret_cast<uint64_t*>(ws + L.sig);
   float* J = reinterpret_cast<float*>(ws + L.J);
   float* Jn = reinterpret_cast<float*>(ws + L.Jn);
   float* sc = reinterpret_cast<float*>(ws + L.sc);
@@ -303,7 +301,6 @@ __device__ __noinline__ void redecide_batch(const NetDesc& net, const State& st,
     }
     if (lane == 0) cnt[q * kMaxL + k] = n | (nn << 16);
     if (k == 0) {
-      if (lane < S) sig[q * S + lane] = word;
       uint64_t zm = lane < S ? zero_mask(word, lane, e_end) : 0ull;
       const int c = __popcll(zm);
       int y = c;
@@ -857,7 +854,7 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
   const int H = net.w[l + 1];
   const bool ahead = i + 1 < H;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gl = lane & (kGroup - 1), grp = lane / kGroup, gsh = lane & kGroup;
+  const int gl = lane & (kGroup - 1), grp = lane / kGroup;
   const long long G = gridDim.x;
   const int32_t* lcur = st.list[n & 1];
   // this group's first splitting edge, loaded together with the counters

@@ -76,7 +76,7 @@ __host__ __device__ inline PtLayout pt_layout(int TV, int mw, int S, int D) {
   const size_t rec = (size_t)TV * p.rows * pt_record(D) * 4;
   p.A = take((size_t)TV * D * D * 4);                 // Newton rows [TV][D][D] (float)
   p.gv = take((size_t)TV * D * 8);                    // their values [TV][D] (double)
-  p.sig = take(0 * (size_t)S);                        // sign words stay in registers
+  p.sig = take(0);                                    // sign words: none, they stay in registers
   p.ahi = take(rec);                                  // records by list position [TV][rows][pt_record]
   // the next layer's, when one pass does not hold all outputs
   p.alo = take(p.rows > kPtRows * pt_lanes(mw, D) ? rec : 0);
@@ -505,19 +505,35 @@ __global__ void __launch_bounds__(kPtThreads, 1) k_polish_rows(NetDesc net, Stat
   if (threadIdx.x == 0 && s_pol) atomic_add_ll(&st.g->polished, static_cast<long long>(s_pol));
 }
 
+// Vertices of a CTA, whether the weights' heads are staged, shared memory and
+// threads of a launch.
+struct PtShape {
+  int TV;
+  bool staged;
+  size_t smem;
+  int threads;
+};
+static PtShape pt_shape(int mw, int S, int D, long long n_params) {
+  PtShape p{};
+  p.TV = pt_tile_vertices(mw, S, D);
+  // the weights' heads beside at least half the vertices, or none
+  const size_t heads = (size_t)(n_params + 3) / 4 * 16;
+  const int least = std::max(4, p.TV / 2);
+  int tv = p.TV;
+  while (tv > least && pt_layout(tv, mw, S, D).total + heads > (size_t)kPtSmemAll) tv -= 4;
+  p.staged = pt_layout(tv, mw, S, D).total + heads <= (size_t)kPtSmemAll;
+  if (p.staged) p.TV = tv;
+  p.smem = pt_layout(p.TV, mw, S, D).total + (p.staged ? heads : 0);
+  p.threads = p.TV * pt_lanes(mw, D);  // whole warps: TV is a multiple of 4
+  return p;
+}
+
 template <int DT, int LN>
 static cudaError_t pt_launch_d(const NetDesc& net, const State& st, float thr, int mw, int num_sms, long long n_params,
                                cudaStream_t stream) {
-  int TV = pt_tile_vertices(mw, net.S, DT);
-  // the weights' heads beside at least half the vertices, or none
-  const size_t heads = (size_t)(n_params + 3) / 4 * 16;
-  const int least = std::max(4, TV / 2);
-  int tv = TV;
-  while (tv > least && pt_layout(tv, mw, net.S, DT).total + heads > (size_t)kPtSmemAll) tv -= 4;
-  const bool staged = pt_layout(tv, mw, net.S, DT).total + heads <= (size_t)kPtSmemAll;
-  if (staged) TV = tv;
-  const size_t smem = pt_layout(TV, mw, net.S, DT).total + (staged ? heads : 0);
-  const int threads = TV * LN;  // whole warps: TV is a multiple of 4
+  const PtShape shape = pt_shape(mw, net.S, DT, n_params);
+  const int TV = shape.TV, threads = shape.threads, staged = shape.staged;
+  const size_t smem = shape.smem;
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_polish_rows<DT, LN>, threads, smem);
   if (e != cudaSuccess) return e;
