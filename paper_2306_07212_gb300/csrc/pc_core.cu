@@ -177,7 +177,15 @@ __global__ void k_init_domain(NetDesc net, State st, const double* X0, const int
 // ---------------------------------------------------------------------------
 // Step (1) at the start of layer l: Z_l = W_l a + b_l for every vertex, with
 // a = x (l = 0) or a_k = z_k of layer l-1 if the vertex's entry is + else 0.
-// SIMT version: one thread per vertex and 16 output neurons per block row.
+// SIMT version: one thread per vertex and 16 output neurons per block row.  It
+// takes every first layer (K = D, in float64), and in float32 the layers that the
+// tensor cores do not (wider than 128) and PC_GEMM_SIMT.  The rows of 128 vertices
+// go through shared memory, 32 inputs at a time and the 16 outputs back, so that
+// reads and writes are coalesced; rows of fewer than 32 floats are read as they
+// lie (most of a row's sectors serve its next inputs from L1).  Products of a
+// whole extraction, a thread reading its own row -> this: 2-256x3-1 net (2.6e5
+// vertices) 3.4 -> 1.9 ms, 3-160x2-1 (4.8e6) 7.9 -> 4.2, 3-64x4-1 0.56 -> 0.30, 5-20x4-1
+// (4.3e5) 0.13 (staged 0.16).
 //
 // FP32 error estimate (root mean square, FP32 and mixed precision): a K-term
 // FP32 dot product accumulated in order has an rms rounding error of about
@@ -199,7 +207,9 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
   }
   const int H = net.w[l + 1], K = net.w[l];
   const int j0 = blockIdx.y * TJ;
-  __shared__ ZT Ws[TJ][kMaxWidth + 1];
+  constexpr int TV = 128, TK = 32;  // vertices and inputs of a staged tile (float32, layers after the first)
+  __shared__ ZT Ws[TJ][(TRACK ? kMaxWidth : kMaxD) + 1];
+  __shared__ float tile[TRACK ? TV : 1][TK + 1];
   __shared__ double Wd[TJ][kMaxD];
   __shared__ ZT bs[TJ];
   __shared__ double bd[TJ];
@@ -219,8 +229,9 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
   const long long Vcap = st.Vcap;
   ZT* Zout = static_cast<ZT*>(st.Z[l]);
   const ZT* Zin = static_cast<const ZT*>(st.Z[l > 0 ? l - 1 : 0]);
-  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < nV;
-       v += (long long)gridDim.x * blockDim.x) {
+  for (long long base = (long long)blockIdx.x * TV; base < nV; base += (long long)gridDim.x * TV) {
+    const long long v = base + threadIdx.x;
+    const bool in = v < nV;
     ZT acc[TJ];
     float a2 = 0.f;
     if (l == 0) {
@@ -228,7 +239,7 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
 #pragma unroll
       for (int jj = 0; jj < TJ; ++jj) dacc[jj] = bd[jj];
       for (int d = 0; d < K; ++d) {
-        const double x = st.X[(long long)d * Vcap + v];
+        const double x = in ? st.X[(long long)d * Vcap + v] : 0.0;
         a2 += static_cast<float>(x * x);
 #pragma unroll
         for (int jj = 0; jj < TJ; ++jj) dacc[jj] = fma(Wd[jj][d], x, dacc[jj]);
@@ -238,19 +249,41 @@ __global__ void __launch_bounds__(128) k_gemm_simt(NetDesc net, State st, int l)
     } else if constexpr (sizeof(ZT) == 4) {  // float64's later layers: k_gemm_f64
 #pragma unroll
       for (int jj = 0; jj < TJ; ++jj) acc[jj] = bs[jj];
-      const ZT* row = Zin + v * K;
-      for (int kk = 0; kk < K; ++kk) {
-        const ZT z = row[kk];
-        const ZT a = z <= ZT(0) ? ZT(0) : z;  // active iff its sign entry is +, iff its value is not <= 0
-        a2 = fmaf(static_cast<float>(a), static_cast<float>(a), a2);
+      auto add = [&](int kk, float a) {
+        a2 = fmaf(a, a, a2);
 #pragma unroll
         for (int jj = 0; jj < TJ; ++jj) acc[jj] = fma(Ws[jj][kk], a, acc[jj]);
+      };
+      auto active = [](float z) { return z <= 0.f ? 0.f : z; };  // iff its sign entry is +, iff its value is not <= 0
+      if (K < TK) {
+        for (int kk = 0; kk < K; ++kk) add(kk, in ? active(Zin[v * K + kk]) : 0.f);
+      } else {
+        for (int k0 = 0; k0 < K; k0 += TK) {
+          const int kk = k0 + threadIdx.x % TK;
+          __syncthreads();  // the tile before has been read
+          for (int r = threadIdx.x / TK; r < TV; r += TV / TK)
+            tile[r][threadIdx.x % TK] = base + r < nV && kk < K ? active(Zin[(base + r) * K + kk]) : 0.f;
+          __syncthreads();
+          const int n = K - k0 < TK ? K - k0 : TK;
+          for (int q = 0; q < n; ++q) add(k0 + q, tile[threadIdx.x][q]);
+        }
       }
     }
+    if constexpr (TRACK) {
+      __syncthreads();
 #pragma unroll
-    for (int jj = 0; jj < TJ; ++jj)
-      if (j0 + jj < H) Zout[v * H + j0 + jj] = acc[jj];
-    if (TRACK && blockIdx.y == 0) {
+      for (int jj = 0; jj < TJ; ++jj) tile[threadIdx.x][jj] = acc[jj];
+      __syncthreads();
+      for (int t = threadIdx.x; t < TV * TJ; t += TV) {
+        const int r = t / TJ, jj = t % TJ;
+        if (base + r < nV && j0 + jj < H) Zout[(base + r) * H + j0 + jj] = tile[r][jj];
+      }
+    } else {
+#pragma unroll
+      for (int jj = 0; jj < TJ; ++jj)
+        if (in && j0 + jj < H) Zout[v * H + j0 + jj] = acc[jj];
+    }
+    if (TRACK && in && blockIdx.y == 0) {
       // rho_l: u/2 ||a||_2 (rounding: the running sums are bounded by
       // ||W_j||_2 ||a||_2) and the largest input error of the previous layer
       const float u = 5.9604645e-8f;  // 2^-24
