@@ -118,10 +118,14 @@ __device__ __forceinline__ bool step_counts(const State& st, int n, long long& n
   return nV >= 0 && nV <= st.Vcap && nE >= 0 && nE <= st.Ecap;
 }
 
-// Entry k of a list.  Each edge is listed at most once, so k < Ecap as long as
-// the step's edges fit (see pair_store for when they do not).
+// How many of the n places from at on lie inside the edge capacity: all of them
+// as long as a step's edges fit (each edge is listed at most once; see
+// warp_flush_pairs for when they do not).
+__device__ __forceinline__ int room(long long at, int n, long long Ecap) {
+  return at + n <= Ecap ? n : at < Ecap ? int(Ecap - at) : 0;
+}
+
 __device__ __forceinline__ void list_store(int32_t* list, long long Ecap, long long k, const ListEntry& x) {
-  if (k >= Ecap) return;
   list[k] = x.e;
   list[Ecap + k] = x.p;
   list[2 * Ecap + k] = x.q;
@@ -135,7 +139,8 @@ __device__ __forceinline__ void warp_flush(const State& st, const ListEntry* la,
   long long base = 0;
   if (lane == 0) base = atomic_add_ll(counter, (long long)lac);
   base = __shfl_sync(0xffffffffu, base, 0);
-  for (int t = lane; t < lac; t += 32) list_store(list, st.Ecap, base + t, la[t]);
+  const int n = room(base, lac, st.Ecap);
+  for (int t = lane; t < n; t += 32) list_store(list, st.Ecap, base + t, la[t]);
   __syncwarp();
   lac = 0;
 }
@@ -746,28 +751,27 @@ __device__ __forceinline__ bool warp_face_matches(const State& st, long long k2,
 // ---------------------------------------------------------------------------
 // One intersecting edge to position x: its record, and its nx (listed at lb
 // + its rank among the listed ones if the next neuron crosses it).
-// The capacity check of a step counts two arrivals at a 2-face, as a generic
-// input has them.  When signs are rounding noise a 2-face can be met more often
-// and every later arrival pairs too (and raises kErrPairing), so x can pass
-// the capacity: such an edge is counted but not stored, and the next kernel
-// that reads the counters finds them above the capacity and stops.
 __device__ __forceinline__ bool pair_splits(const int4& rec) { return (rec.w ^ (rec.w >> 1)) & 1; }
 
 __device__ __forceinline__ void pair_store(const State& st, long long x, const int4& rec, int n, bool ahead,
                                            int32_t* lnext, long long at) {
-  if (x >= st.Ecap) return;
   st.EU[x] = rec.x;
   st.EW[x] = rec.y;
   if (st.deferred) st.vlist[x] = make_int4(rec.x, rec.y, rec.z, n + 1);
   if (!ahead) return;
   const bool hit = pair_splits(rec);
   st.nx[x] = hit ? kNxListed : kNxFresh;
-  if (hit)
+  if (hit && at < st.Ecap)
     list_store(lnext, st.Ecap, at, (rec.w & 1) ? ListEntry{int(x), rec.y, rec.x} : ListEntry{int(x), rec.x, rec.y});
 }
 
 // Appends the warp's buffered intersecting edges (pc, of them pla that split
 // at the next neuron) with one atomic each.
+// The capacity check of a step counts two arrivals at a 2-face, as a generic
+// input has them.  When signs are rounding noise a 2-face can be met more often
+// and every later arrival pairs too (and raises kErrPairing), so the edges can
+// pass the capacity: those are counted but not stored, and the next kernel that
+// reads the counters finds them above the capacity and stops.
 __device__ __forceinline__ void warp_flush_pairs(const State& st, const int4* pairs, int& pc, int& pla, Counters* cur,
                                                  long long* cnext, int32_t* lnext, long long ebase, int n,
                                                  bool ahead) {
@@ -778,8 +782,9 @@ __device__ __forceinline__ void warp_flush_pairs(const State& st, const int4* pa
   if (lane == 1 && ahead && pla) lb = atomic_add_ll(cnext, (long long)pla);
   pb = ebase + __shfl_sync(0xffffffffu, pb, 0);
   lb = __shfl_sync(0xffffffffu, lb, 1);
-  for (int t0 = 0; t0 < pc; t0 += 32) {
-    const bool in = t0 + lane < pc;
+  const int np = room(pb, pc, st.Ecap);
+  for (int t0 = 0; t0 < np; t0 += 32) {
+    const bool in = t0 + lane < np;
     const int4 rec = in ? pairs[t0 + lane] : make_int4(0, 0, 0, 0);
     const unsigned b = __ballot_sync(0xffffffffu, in && ahead && pair_splits(rec));
     if (in) pair_store(st, pb + t0 + lane, rec, n, ahead, lnext, lb + __popc(b & ((1u << lane) - 1u)));
@@ -818,11 +823,11 @@ __device__ void flush_cta(const State& st, Counters* cur, long long* cnext, int3
   __syncthreads();
   const long long pb = ebase + sm.pbase + fa;
   long long lb = sm.lbase + fb;
-  if (ahead)
-    for (int t = lane; t < lac; t += 32) list_store(lnext, st.Ecap, lb + t, sm.la[warp][t]);
+  const int nl = ahead ? room(lb, lac, st.Ecap) : 0, np = room(pb, pc, st.Ecap);
+  for (int t = lane; t < nl; t += 32) list_store(lnext, st.Ecap, lb + t, sm.la[warp][t]);
   lb += lac;
-  for (int t0 = 0; t0 < pc; t0 += 32) {
-    const bool in = t0 + lane < pc;
+  for (int t0 = 0; t0 < np; t0 += 32) {
+    const bool in = t0 + lane < np;
     const int4 rec = in ? sm.pairs[warp][t0 + lane] : make_int4(0, 0, 0, 0);
     const unsigned hb = __ballot_sync(0xffffffffu, in && ahead && pair_splits(rec));
     if (in) pair_store(st, pb + t0 + lane, rec, n, ahead, lnext, lb + __popc(hb & ((1u << lane) - 1u)));
