@@ -172,14 +172,12 @@ __global__ void __launch_bounds__(512) k_adj_wgrad(NetDesc net, State st, const 
 // consecutive threads take consecutive k, so weights and rows are coalesced and
 // zbar_l[v][j] is one broadcast.  A weight is a float pair too; the remainders are
 // read only for a network that has any (NetDesc::rem).
-template <typename ZT>
-__global__ void __launch_bounds__(256) k_adj_back(NetDesc net, State st, const double* zbar, double* zprev, int l,
-                                                  long long nVl) {
-  extern __shared__ float2 sh[];  // [kAdjTile][H]
+template <typename ZT, bool PAIRS>
+__device__ __forceinline__ void adj_back(const NetDesc& net, const State& st, const double* zbar, double* zprev, int l,
+                                         long long nVl, float2* sh) {
   const int H = net.w[l + 1], K = net.w[l];
   const float* W = net.W32 + net.wofs[l];
   const float* R = net.R32 + net.wofs[l];
-  const bool pairs = *net.rem != 0;
   const ZT* Zin = static_cast<const ZT*>(st.Z[l - 1]);
   for (long long base = (long long)blockIdx.x * kAdjTile; base < nVl; base += (long long)gridDim.x * kAdjTile) {
     const int n = nVl - base < kAdjTile ? int(nVl - base) : kAdjTile;
@@ -188,17 +186,21 @@ __global__ void __launch_bounds__(256) k_adj_back(NetDesc net, State st, const d
     for (int t = threadIdx.x; t < n * K; t += blockDim.x) {
       const int c = t / K, k = t - c * K;
       float s = 0.f, e = 0.f;
-      if (!(Zin[base * K + t] <= ZT(0))) {  // active iff its sign entry is +
-        if (pairs)
-          for (int j = 0; j < H; ++j)
-            dot2(sh[c * H + j], make_float2(W[(long long)j * K + k], R[(long long)j * K + k]), s, e);
-        else
-          for (int j = 0; j < H; ++j) dot2(sh[c * H + j], make_float2(W[(long long)j * K + k], 0.f), s, e);
-      }
+      if (!(Zin[base * K + t] <= ZT(0)))  // active iff its sign entry is +
+        for (int j = 0; j < H; ++j)
+          dot2(sh[c * H + j], make_float2(W[(long long)j * K + k], PAIRS ? R[(long long)j * K + k] : 0.f), s, e);
       zprev[base * K + t] = static_cast<double>(s) + static_cast<double>(e);
     }
     __syncthreads();
   }
+}
+
+template <typename ZT>
+__global__ void __launch_bounds__(256) k_adj_back(NetDesc net, State st, const double* zbar, double* zprev, int l,
+                                                  long long nVl) {
+  extern __shared__ float2 sh[];  // [kAdjTile][H]
+  if (*net.rem) adj_back<ZT, true>(net, st, zbar, zprev, l, nVl, sh);
+  else adj_back<ZT, false>(net, st, zbar, zprev, l, nVl, sh);
 }
 
 template <typename ZT>
