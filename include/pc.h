@@ -387,8 +387,8 @@ pc_status pc_server_destroy(pc_server *s);
  * Blocks until done.
  *
  * Alignment: cap_e must be a multiple of 4 and E must start on a 16-byte
- * boundary (the edge pass reads both endpoint rows with 16-byte loads); X
- * and SIG must be 8-byte aligned.  Otherwise the call returns PC_ERR_INVALID
+ * boundary (so that both endpoint rows do); X and SIG must be 8-byte
+ * aligned.  Otherwise the call returns PC_ERR_INVALID
  * before any device work.
  *
  * All other working memory is one static device array of about 15 MB

@@ -171,8 +171,10 @@ class Extractor:
     """One libpc context: extract complexes of ReLU MLPs on a box.
 
     precision: "fp32" | "mixed" (FP32 bulk, FP64 re-evaluation of signs within
-    the FP32 error bound) | "fp64".  execution: "persistent" (one cooperative
-    kernel per layer) | "stepwise" (one kernel per step and neuron).
+    the FP32 error bound) | "fp64".  execution: "persistent" (one kernel per
+    layer: cooperative, or one thread-block cluster while small) | "stepwise"
+    (no grid barrier: one cluster per layer while small, else one kernel per
+    step and neuron).
     max_dim: the largest input dimension the context takes, 8 (libpc.so) or
     10 (libpc_d10.so, the same kernels with larger per-vertex arrays).
     debug_barrier_timeout: testing only; the persistent kernel's grid barriers

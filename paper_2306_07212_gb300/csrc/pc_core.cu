@@ -569,8 +569,8 @@ static size_t zsize_of(int prec) { return prec == PC_PREC_FP64 ? 8 : 4; }
 // are (re)shaped), which covers every network that runs without reshaping,
 // not from the current network (a later, wider one would overrun them).
 static void realloc_state(pc_ctx* c, long long V, long long E, long long T, bool copy) {
-  // multiples of 64 entries: rows stay 256-byte aligned (vector loads of the
-  // second endpoint row need EW = EU + Ecap on a 16-byte boundary)
+  // multiples of 64 entries: every row starts on a 256-byte boundary (whole
+  // sectors; the scan reads nx 16 bytes at a time, up to 14 bytes past the count)
   V = std::min<long long>((V + 63) & ~63ll, (1ll << 31) - 64);
   E = std::min<long long>((E + 63) & ~63ll, (1ll << 31) - 64);
   const int D = c->shape_D, S = c->shape_S, Hm = c->shape_H;
@@ -747,6 +747,10 @@ static int cluster_ctas(const pc_ctx* c) {
   else if (shares_gpu(c) || c->Ecap > kClusterE) small = c->Ecap <= kClusterE;
   else small = (c->net.fA ? double(c->Vcap) : std::min(double(c->Vcap), most_vertices(c->net))) <= double(kAloneV);
   if (!small) return 0;
+  // 16 where a step has more splits than 8 CTAs hold (256), by the capacity per
+  // neuron: a 4-8x3-1 net (9.5e3 vertices) 0.62 ms and 0.77 with 8, a 2-40x4-1 net
+  // 2.17 and 2.22; a 1-40x10-1 net (357 vertices, float64) 2.70 and 2.65.  Between
+  // them the line is not sharp (a 2-64x10-1 window, 51 per neuron: 9.0 and 10.8).
   return c->big_cluster && c->Vcap > 64ll * c->N ? 16 : 8;
 }
 
@@ -1666,8 +1670,7 @@ extern "C" pc_status pc_extract_noalloc(int L, const int32_t* widths, const doub
   if (n > kNaMaxN || p > kNaMaxParams || 2 * D + n > kMaxEntries) return PC_ERR_TOO_LARGE;
   if (cap_v > kNaMaxV || cap_e > kNaMaxE) return PC_ERR_TOO_LARGE;
   if (cap_v < (1 << D) || cap_e < (long long)D << (D - 1)) return PC_ERR_INVALID;
-  // the edge pass reads four endpoints at a time with 16-byte loads from E and
-  // from its second row E + cap_e: both must sit on 16-byte boundaries
+  // the call's contract (pc.h); X and SIG are read as 8-byte words
   if (cap_e % 4 != 0 || (reinterpret_cast<uintptr_t>(E) & 15) || (reinterpret_cast<uintptr_t>(X) & 7) ||
       (reinterpret_cast<uintptr_t>(SIG) & 7))
     return PC_ERR_INVALID;

@@ -845,8 +845,9 @@ __device__ void flush_cta(const State& st, Counters* cur, long long* cnext, int3
 // chains in flight.  So half a warp takes a split: the values lie vertex by
 // vertex, 16 lanes read a row of 64 floats with four coalesced loads, every
 // reduction has four shuffle steps for two splits at once, and 16 warps with
-// up to 128 registers a thread keep 32 splits per SM in flight without
-// spilling.
+// up to 128 registers a thread keep 32 splits per SM in flight.  The mixed form,
+// which also carries the queue of re-decisions, spills at that (k_layer: 354 bytes
+// of stores and 540 of loads a thread), the others less (24 to 68 of stores).
 // Measured on GB300 against a warp per split, values neuron by neuron and two
 // CTAs of 512 threads with 64 registers: neuron loop of a 5-40x4-1 net (1e7
 // vertices) 63.4 -> 36.5 ms, of an 8-10x4-1 net 2.8 -> 1.9 ms, of a 3-64x4-1
@@ -1359,7 +1360,8 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
             // scale takes the endpoints' (a convex combination does not amplify
             // them) and the interpolation's rounding (u |z_j|, in units of
             // ||W_j||_2); the position takes the endpoints' estimates and the
-            // shift along the edge that the errors of a and b cause in t.
+            // shift along the edge that the errors of a and b cause in t (all in
+            // float32: estimates).
             const float rm = fmaxf(rp, rq_), rr_ = 5.9604645e-8f * amax;
             esc0 = sqrtf(rm * rm + rr_ * rr_);
             st.esc[v0] = esc0;
@@ -1400,7 +1402,7 @@ __device__ bool phase_step(const NetDesc& net, const State& st, int l, int i, Sm
           if (MIXED && pend) {
             const int x = atomicAdd(&sm.npend, 1);  // < kPendCap: looked at every kPendRounds rounds
             sm.pend.split.v0[x] = v0;
-              sm.pend.split.k[x] = bad ? ~k : k;
+            sm.pend.split.k[x] = bad ? ~k : k;
           }
         }
         ready = okA && !pend;

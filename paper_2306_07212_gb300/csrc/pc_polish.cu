@@ -17,14 +17,18 @@
 // one or two 16-byte broadcasts from shared memory) serves up to 64 outputs,
 // and pairs of outputs run on packed FP32 instructions (each rounded as the
 // scalar form).  Weight heads are staged in shared memory when they fit; their
-// remainders are read only for networks that have any (NetDesc::rem).
+// remainders are read only for networks that have any (NetDesc::rem); such a
+// network's pairs come from global memory: 3-64x3-1 net (8.9e5 vertices) 1.69 ms
+// staged and 1.93 as pairs, 5-30x3-1 (2.1e6) 2.66 and 3.31.
 //
 // The dot products follow Ogita-Rump-Oishi Dot2 (exact products by FMA, TwoSum
 // of the running sum, error terms summed in a float), about 44 bits; a skipped
 // zero input changes no bit of them, so every sum is the dense one's in its
 // order.
 //
-// Bound by FP32 issue.  Measured on GB300 against a dense product over tiles
+// Bound by FP32 issue.  The instances take all 128 registers of the launch bound
+// and spill, more with D: 84 bytes of stores and 172 of loads a thread at D = 3,
+// 352 and 500 at D = 5, 404 and 1180 at D = 8 (8 lanes).  Measured on GB300 against a dense product over tiles
 // of 32 vertices (D <= 5) and a dense pass of a warp per vertex (D > 5):
 // 3-64x4-1 (314k vertices) 2.57 -> 0.77 ms, 5-40x4-1 (1e7) 39 -> 15.7 ms,
 // 4-128x3-1 (212k) 3.8 -> 1.35 ms, 8-10x4-1 (369k) 7.7 -> 0.93 ms.

@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kCompactBlock) k_edge_scatter(State st, const 
 }
 
 // Copies the compacted edges back and records the pruned count for the
-// next step (read by phase_classify as the edge count after this layer).
+// next step (step_counts reads it as the edge count after this layer).
 __global__ void k_edge_commit(State st, Counters* cn, const int* total, const int32_t* tU, const int32_t* tW,
                               const int4* tL) {
   if (g_stopped(st.g)) return;
