@@ -118,13 +118,6 @@ __device__ __forceinline__ bool step_counts(const State& st, int n, long long& n
   return nV >= 0 && nV <= st.Vcap && nE >= 0 && nE <= st.Ecap;
 }
 
-// How many of the n places from at on lie inside the edge capacity: all of them
-// as long as a step's edges fit (each edge is listed at most once; see
-// warp_flush_pairs for when they do not).
-__device__ __forceinline__ int room(long long at, int n, long long Ecap) {
-  return at + n <= Ecap ? n : at < Ecap ? int(Ecap - at) : 0;
-}
-
 __device__ __forceinline__ void list_store(int32_t* list, long long Ecap, long long k, const ListEntry& x) {
   list[k] = x.e;
   list[Ecap + k] = x.p;
@@ -139,8 +132,8 @@ __device__ __forceinline__ void warp_flush(const State& st, const ListEntry* la,
   long long base = 0;
   if (lane == 0) base = atomic_add_ll(counter, (long long)lac);
   base = __shfl_sync(0xffffffffu, base, 0);
-  const int n = room(base, lac, st.Ecap);
-  for (int t = lane; t < n; t += 32) list_store(list, st.Ecap, base + t, la[t]);
+  if (base + lac <= st.Ecap)  // see warp_flush_pairs
+    for (int t = lane; t < lac; t += 32) list_store(list, st.Ecap, base + t, la[t]);
   __syncwarp();
   lac = 0;
 }
@@ -761,7 +754,7 @@ __device__ __forceinline__ void pair_store(const State& st, long long x, const i
   if (!ahead) return;
   const bool hit = pair_splits(rec);
   st.nx[x] = hit ? kNxListed : kNxFresh;
-  if (hit && at < st.Ecap)
+  if (hit)
     list_store(lnext, st.Ecap, at, (rec.w & 1) ? ListEntry{int(x), rec.y, rec.x} : ListEntry{int(x), rec.x, rec.y});
 }
 
@@ -770,8 +763,9 @@ __device__ __forceinline__ void pair_store(const State& st, long long x, const i
 // The capacity check of a step counts two arrivals at a 2-face, as a generic
 // input has them.  When signs are rounding noise a 2-face can be met more often
 // and every later arrival pairs too (and raises kErrPairing), so the edges can
-// pass the capacity: those are counted but not stored, and the next kernel that
-// reads the counters finds them above the capacity and stops.
+// pass the capacity, and with them the list (each edge is listed at most once).
+// Entries whose places are not all inside are counted but not stored, and the
+// next kernel that reads the counters finds them above the capacity and stops.
 __device__ __forceinline__ void warp_flush_pairs(const State& st, const int4* pairs, int& pc, int& pla, Counters* cur,
                                                  long long* cnext, int32_t* lnext, long long ebase, int n,
                                                  bool ahead) {
@@ -782,7 +776,7 @@ __device__ __forceinline__ void warp_flush_pairs(const State& st, const int4* pa
   if (lane == 1 && ahead && pla) lb = atomic_add_ll(cnext, (long long)pla);
   pb = ebase + __shfl_sync(0xffffffffu, pb, 0);
   lb = __shfl_sync(0xffffffffu, lb, 1);
-  const int np = room(pb, pc, st.Ecap);
+  const int np = pb + pc <= st.Ecap && lb + pla <= st.Ecap ? pc : 0;
   for (int t0 = 0; t0 < np; t0 += 32) {
     const bool in = t0 + lane < np;
     const int4 rec = in ? pairs[t0 + lane] : make_int4(0, 0, 0, 0);
@@ -817,17 +811,20 @@ __device__ void flush_cta(const State& st, Counters* cur, long long* cnext, int3
     long long x = 0, y = 0;
     if (na) x = atomic_add_ll(&cur->npairs, (long long)na);
     if (ahead && nb) y = atomic_add_ll(cnext, (long long)nb);
+    if (ebase + x + na > st.Ecap || y + nb > st.Ecap) x = -1;  // nothing stored (see warp_flush_pairs)
     sm.pbase = x;
     sm.lbase = y;
   }
   __syncthreads();
-  const long long pb = ebase + sm.pbase + fa;
+  long long pb = sm.pbase;
+  if (pb < 0) return;  // uniform
+  pb += ebase + fa;
   long long lb = sm.lbase + fb;
-  const int nl = ahead ? room(lb, lac, st.Ecap) : 0, np = room(pb, pc, st.Ecap);
-  for (int t = lane; t < nl; t += 32) list_store(lnext, st.Ecap, lb + t, sm.la[warp][t]);
+  if (ahead)
+    for (int t = lane; t < lac; t += 32) list_store(lnext, st.Ecap, lb + t, sm.la[warp][t]);
   lb += lac;
-  for (int t0 = 0; t0 < np; t0 += 32) {
-    const bool in = t0 + lane < np;
+  for (int t0 = 0; t0 < pc; t0 += 32) {
+    const bool in = t0 + lane < pc;
     const int4 rec = in ? sm.pairs[warp][t0 + lane] : make_int4(0, 0, 0, 0);
     const unsigned hb = __ballot_sync(0xffffffffu, in && ahead && pair_splits(rec));
     if (in) pair_store(st, pb + t0 + lane, rec, n, ahead, lnext, lb + __popc(hb & ((1u << lane) - 1u)));
@@ -846,8 +843,8 @@ __device__ void flush_cta(const State& st, Counters* cur, long long* cnext, int3
 // vertex, 16 lanes read a row of 64 floats with four coalesced loads, every
 // reduction has four shuffle steps for two splits at once, and 16 warps with
 // up to 128 registers a thread keep 32 splits per SM in flight.  The mixed form,
-// which also carries the queue of re-decisions, spills at that (k_layer: 354 bytes
-// of stores and 540 of loads a thread), the others less (24 to 68 of stores).
+// which also carries the queue of re-decisions, spills at that (k_layer: 358 bytes
+// of stores and 560 of loads a thread), the others less (up to 48 of stores).
 // Measured on GB300 against a warp per split, values neuron by neuron and two
 // CTAs of 512 threads with 64 registers: neuron loop of a 5-40x4-1 net (1e7
 // vertices) 63.4 -> 36.5 ms, of an 8-10x4-1 net 2.8 -> 1.9 ms, of a 3-64x4-1
