@@ -43,14 +43,17 @@ __device__ inline void domain_facet_rows(const NetDesc& net, const State& st, lo
   s_zl[q] = j + kFacetRow;
 }
 
-// The system M x = r in float32 by one warp (lane r < D: row r of M and its
-// right-hand side; all lanes call it): Gauss-Jordan elimination with partial
-// pivoting.  Component d of the solution in lane d.  False when singular.
-__device__ inline bool solve_warp(int D, const float (&A)[kMaxD], float rhs, float& x) {
+// The inverse of M in float32 by one warp (lane r < D: row r of M; all lanes call
+// it): Gauss-Jordan elimination of [M | I] with partial pivoting.  Row c of the
+// inverse in lane c.  False when singular.
+__device__ inline bool invert_warp(int D, const float (&A)[kMaxD], float (&V)[kMaxD]) {
   const int lane = threadIdx.x & 31;
   float M[kMaxD];
 #pragma unroll
-  for (int c = 0; c < kMaxD; ++c) M[c] = A[c];
+  for (int c = 0; c < kMaxD; ++c) {
+    M[c] = A[c];
+    V[c] = lane == c ? 1.f : 0.f;
+  }
   int var = -1;  // the column whose pivot this lane's row is
   float diag = 1.f;
 #pragma unroll
@@ -69,15 +72,19 @@ __device__ inline bool solve_warp(int D, const float (&A)[kMaxD], float rhs, flo
 #pragma unroll
     for (int k = 0; k < kMaxD; ++k)
       if (k > c && k < D) M[k] -= f * __shfl_sync(0xffffffffu, M[k], piv);
-    rhs -= f * __shfl_sync(0xffffffffu, rhs, piv);
+#pragma unroll
+    for (int k = 0; k < kMaxD; ++k)
+      if (k < D) V[k] -= f * __shfl_sync(0xffffffffu, V[k], piv);
   }
-  const float mine = rhs / diag;
-  x = 0.f;
+  const float inv = 1.f / diag;
+  int from = lane;
   for (int c = 0; c < D; ++c) {
     const int src = __ffs(__ballot_sync(0xffffffffu, var == c)) - 1;
-    const float y = __shfl_sync(0xffffffffu, mine, src);
-    if (lane == c) x = y;
+    if (lane == c) from = src;
   }
+#pragma unroll
+  for (int k = 0; k < kMaxD; ++k)
+    if (k < D) V[k] = __shfl_sync(0xffffffffu, V[k] * inv, from);
   return true;
 }
 
@@ -153,16 +160,17 @@ static __device__ __noinline__ bool newton_warp64(const NetDesc& net, const Stat
 
 // The same step by one warp (all lanes call it; the zero set has D entries) to
 // the accuracy of an elimination in float64, which took 9,500 clocks at D = 3
-// (a float64 division takes ~2000 on this chip): a float32 solve, then float32
-// corrections of its residual, which is formed in float64 (iterative
-// refinement: a correction is about rho times the one before, rho ~ condition
-// number x 2^-24).  Two corrections do for condition numbers up to a few
-// hundred: the second is then below 2^-29 of the step, and what is left, rho x
-// 2^-29, below what the elimination's own rounding leaves (condition number x
-// 2^-53).  More are made until that holds.  A system whose corrections do not
-// halve, or would take more than kNewtonSolves solves (rho above ~1/6), or that
-// is singular in float32 is eliminated in float64.  dl: component of the step
-// in lane d < D.  False when the system is singular.
+// (a float64 division takes ~2000 on this chip): float32 solves, by one inverse,
+// of residuals formed in float64 (iterative refinement: a correction is about rho
+// times the one before, rho ~ condition number x 2^-24).  Two corrections do for
+// condition numbers up to a few hundred: the second is then below 2^-29 of the
+// step, and what is left, rho x 2^-29, below what the elimination's own rounding
+// leaves (condition number x 2^-53).  More are made until that holds.  A system
+// whose corrections do not halve, or would take more than kNewtonSolves solves (rho
+// above ~1/6), or that is singular in float32 is eliminated in float64.  dl:
+// component of the step in lane d < D.  False when the system is singular.
+// An elimination per solve instead of the inverse: neuron loop of a 3-64x4-1 net
+// 5.25 ms, so 5.11 (5.18 with two corrections and no look at them).
 constexpr int kNewtonSolves = 12;
 
 __device__ inline bool newton_warp(const NetDesc& net, const State& st, long long v, const int* s_zl, const double* A,
@@ -178,11 +186,17 @@ __device__ inline bool newton_warp(const NetDesc& net, const State& st, long lon
   const double scale = top > 0 && top < 2046 ? __hiloint2double((2046 - top) << 20, 0) : 1.0;
 #pragma unroll
   for (int c = 0; c < kMaxD; ++c) F[c] = static_cast<float>(M[c] * scale);
+  float V[kMaxD];
+  if (!invert_warp(D, F, V)) return newton_warp64(net, st, v, s_zl, A, gv, dl);
   dl = 0.0;
   float first = 0.f, before = 0.f;  // the largest components of the first solve and of the last one
   for (int it = 0; it < kNewtonSolves; ++it) {
-    float x;
-    if (!solve_warp(D, F, static_cast<float>(r * scale), x)) break;
+    const float rf = static_cast<float>(r * scale);
+    float x = 0.f;
+#pragma unroll
+    for (int c = 0; c < kMaxD; ++c)
+      if (c < D) x = fmaf(V[c], __shfl_sync(0xffffffffu, rf, c), x);
+    if ((threadIdx.x & 31) >= D) x = 0.f;
     dl += static_cast<double>(x);
     const float size = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(x))));
     if (it == 0) first = size;
