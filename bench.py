@@ -49,8 +49,8 @@ sys.path.insert(0, ROOT)
 #   k_layer_torus      the D=3 torus workload, 5 k_layer launches
 #   k_layer_d5w40      the D=5 width-40 counting-sweep net (seed 0), 5 launches
 #   k_gemm_tc2_d5w40   the same net's 4 tensor-core layer products
-KERNEL_DRAM = {"sources_sha16": "c2e35648be02bf0d", "k_layer_torus": 42841600, "k_layer_d5w40": 9383006618,
-               "k_gemm_tc2_d5w40": 1464939584}
+KERNEL_DRAM = {"sources_sha16": "1f8aca7266bf5227", "k_layer_torus": 43916698, "k_layer_d5w40": 9431827507,
+               "k_gemm_tc2_d5w40": 1465161472}
 KERNEL_SOURCES = ("pc_phases.cuh", "pc_core.cu", "pc_device.cuh", "pc_newton.cuh", "pc_gemm_tc.cu", "pc_polish.cu")
 
 METRIC = "vertices+edges/s at D=3 (torus 3-64x4-1, box [-1,1]^3)"
